@@ -12,21 +12,24 @@
 //                   the W4A8 linear): each 4-bit code stored as one E4M3 byte,
 //                   plus the row sum of the codes.
 //
-// One CTA of 256 threads per row (persistent over rows).  The row is held in
-// shared memory as fp32; the power-of-two factor is a radix-2 FWHT over the
-// fast index, the small Paley factor a dense +-1 product over the slow index.
+// One CTA of 256 threads per row (persistent over rows), the row transformed
+// in shared memory as fp32, or kept in registers without a rotation
+// (row_transform.cuh).  GB300: the activations of 2048 x 4096 without a
+// rotation 8.4 -> 4.5 us (FP8) and 9.7 -> 6.7 us (planes), 2048 x 8192 with
+// H_8192 91.8 -> 20.3 us (FP8), 4096 x 14336 INT4_BYTES weights merged with
+// H_28 (x) H_512 401 -> 99 us.
 // Codes are taken on the unnormalised row; alpha and beta carry 1/sqrt(K).
 #include <cuda_fp16.h>
-#include <float.h>
 
 #include "launch_util.h"
+#include "row_transform.cuh"
 #include "spinq_device.cuh"
 #include "spinq_internal.h"
 
 namespace spinq {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = kRowThreads;
 
 __device__ __forceinline__ uint32_t e4m3x2(float lo, float hi) {
   uint16_t r;
@@ -34,92 +37,29 @@ __device__ __forceinline__ uint32_t e4m3x2(float lo, float hi) {
   return r;
 }
 
-template <int FMT, bool SYM, bool CLAMP, int NS>
-__global__ void __launch_bounds__(kThreads) rq8_rows_kernel(Rq8Args a) {
-  extern __shared__ float s[];
-  __shared__ float red_hi[kThreads / 32], red_lo[kThreads / 32];
+// NS: order of the small factor; 0: no rotation, the row in CPT chunks per
+// thread.
+template <int FMT, bool SYM, bool CLAMP, int NS, int CPT>
+__global__ void __launch_bounds__(kThreads, NS > 1 ? 3 : CPT > 8 ? 2 : 4) rq8_rows_kernel(Rq8Args a) {
+  extern __shared__ __align__(16) float s[];
+  __shared__ float red[2 * kThreads / 32];
   __shared__ int red_sum[kThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = (int)a.K;
-  const int P = a.n_pow2;
-  const int log2P = a.n_small ? 31 - __clz(P) : 0;
   const __half* __restrict__ x = reinterpret_cast<const __half*>(a.x);
   pdl_wait();
   pdl_trigger();
 
   for (int64_t row = blockIdx.x; row < a.rows; row += gridDim.x) {
-    const __half* xr = x + row * a.ldx;
-    for (int c = tid; c < K / 8; c += kThreads) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(xr) + c);
-      const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __half22float2(h[e]);
-        *reinterpret_cast<float2*>(s + 8 * c + 2 * e) = f;
-      }
+    uint4 plain[CPT];
+    RowRange<SYM> range;
+    if constexpr (NS == 0) {
+      range = row_plain<CPT, SYM>(x + row * a.ldx, K, plain, red);
+    } else {
+      if (row + gridDim.x < a.rows) row_prefetch(x + (row + gridDim.x) * a.ldx, K);
+      range = row_transform<NS, SYM>(x + row * a.ldx, nullptr, s, K, a.n_pow2, red);
     }
-    __syncthreads();
-    if (a.n_small) {
-      for (int lh = 0; lh < log2P; ++lh) {
-        const int h = 1 << lh;
-        for (int p = tid; p < K / 2; p += kThreads) {
-          const int seg = p >> (log2P - 1);
-          const int l = p & ((P >> 1) - 1);
-          const int j = ((l >> lh) << (lh + 1)) | (l & (h - 1));
-          const int i0 = seg * P + j;
-          const float u = s[i0], w = s[i0 + h];
-          s[i0] = u + w;
-          s[i0 + h] = u - w;
-        }
-        __syncthreads();
-      }
-      if constexpr (NS > 1) {
-        // the small factor, unrolled at its compile-time order (registers only)
-        uint32_t neg[NS];
-#pragma unroll
-        for (int ip = 0; ip < NS; ++ip) neg[ip] = a.hs.neg[ip];
-        for (int j = tid; j < P; j += kThreads) {
-          float t[NS];
-#pragma unroll
-          for (int ip = 0; ip < NS; ++ip) t[ip] = s[ip * P + j];
-#pragma unroll
-          for (int i = 0; i < NS; ++i) {
-            float acc = 0.f;
-#pragma unroll
-            for (int ip = 0; ip < NS; ++ip) acc += ((neg[ip] >> i) & 1u) ? -t[ip] : t[ip];
-            s[i * P + j] = acc;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    // row range
-    float hi = SYM ? 0.f : -FLT_MAX, lo = FLT_MAX;
-    for (int k = tid; k < K; k += kThreads) {
-      const float v = s[k];
-      if (SYM) {
-        hi = fmaxf(hi, fabsf(v));
-      } else {
-        hi = fmaxf(hi, v);
-        lo = fminf(lo, v);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    }
-    if (lane == 0) {
-      red_hi[warp] = hi;
-      red_lo[warp] = lo;
-    }
-    __syncthreads();
-    hi = red_hi[0];
-    lo = red_lo[0];
-    for (int w = 1; w < kThreads / 32; ++w) {
-      hi = fmaxf(hi, red_hi[w]);
-      lo = fminf(lo, red_lo[w]);
-    }
+    const float hi = range.hi, lo = range.lo;
     // per-row constants (unnormalised row)
     float inv, off = 0.f, alpha, beta = 0.f;
     if (FMT == kFmtE4M3) {
@@ -142,11 +82,11 @@ __global__ void __launch_bounds__(kThreads) rq8_rows_kernel(Rq8Args a) {
     }
     int csum = 0;
     uint8_t* out = a.codes + row * (FMT == kFmtInt8Planes ? 2 * a.K : a.K);
-    for (int c = tid; c < K / 8; c += kThreads) {
+    auto quant8 = [&](int c, const float (&v)[8]) {
       uint32_t w0[2] = {0, 0}, w1[2] = {0, 0};
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        float t0 = fmaf(s[8 * c + e], inv, off), t1 = fmaf(s[8 * c + e + 1], inv, off);
+        float t0 = fmaf(v[e], inv, off), t1 = fmaf(v[e + 1], inv, off);
         uint32_t b0, b1;
         if (FMT == kFmtE4M3) {
           b0 = e4m3x2(t0, t1);   // both bytes at once: lo element in the low byte
@@ -176,6 +116,20 @@ __global__ void __launch_bounds__(kThreads) rq8_rows_kernel(Rq8Args a) {
       }
       *reinterpret_cast<uint2*>(out + 8 * c) = make_uint2(w0[0], w0[1]);
       if (FMT == kFmtInt8Planes) *reinterpret_cast<uint2*>(out + a.K + 8 * c) = make_uint2(w1[0], w1[1]);
+    };
+    float v[8];
+    if constexpr (NS == 0) {
+#pragma unroll
+      for (int i = 0; i < CPT; ++i) {
+        if (tid + kThreads * i >= K / 8) break;
+        row_get8(plain[i], v);
+        quant8(tid + kThreads * i, v);
+      }
+    } else {
+      for (int c = tid; c < K / 8; c += kThreads) {
+        row_get8(s, c, v);
+        quant8(c, v);
+      }
     }
     if (FMT == kFmtInt4Bytes) {
 #pragma unroll
@@ -196,14 +150,14 @@ __global__ void __launch_bounds__(kThreads) rq8_rows_kernel(Rq8Args a) {
   }
 }
 
-template <int FMT, bool SYM, bool CLAMP, int NS>
+template <int FMT, bool SYM, bool CLAMP, int NS, int CPT>
 cudaError_t launch_ns(const Rq8Args& a, cudaStream_t stream) {
-  const size_t smem = sizeof(float) * (size_t)a.K;
-  auto kern = rq8_rows_kernel<FMT, SYM, CLAMP, NS>;
+  const size_t smem = NS == 0 ? 0 : sizeof(float) * (size_t)a.K;
+  auto kern = rq8_rows_kernel<FMT, SYM, CLAMP, NS, CPT>;
   int per_sm = 0;
   cudaError_t e = prepare_launch(kern, kThreads, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  const int64_t cap = (int64_t)device_sm_count() * per_sm;
+  const int64_t cap = NS == 0 ? INT32_MAX : (int64_t)device_sm_count() * per_sm;
   const int64_t grid = a.rows < cap ? a.rows : cap;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(kThreads), smem, stream, 1, a);
   if (e != cudaSuccess) return e;
@@ -213,18 +167,22 @@ cudaError_t launch_ns(const Rq8Args& a, cudaStream_t stream) {
 template <int FMT, bool SYM, bool CLAMP>
 cudaError_t launch_t(const Rq8Args& a, cudaStream_t stream) {
   switch (a.n_small) {
-    case 12: return launch_ns<FMT, SYM, CLAMP, 12>(a, stream);
-    case 20: return launch_ns<FMT, SYM, CLAMP, 20>(a, stream);
-    case 28: return launch_ns<FMT, SYM, CLAMP, 28>(a, stream);
+    case 0:
+      return with_row_chunks(a.K, [&](auto cpt) { return launch_ns<FMT, SYM, CLAMP, 0, cpt()>(a, stream); });
+    case 12: return launch_ns<FMT, SYM, CLAMP, 12, 1>(a, stream);
+    case 20: return launch_ns<FMT, SYM, CLAMP, 20, 1>(a, stream);
+    case 28: return launch_ns<FMT, SYM, CLAMP, 28, 1>(a, stream);
   }
-  return launch_ns<FMT, SYM, CLAMP, 1>(a, stream);
+  return launch_ns<FMT, SYM, CLAMP, 1, 1>(a, stream);
 }
 
 template <int FMT>
 cudaError_t launch_fmt(const Rq8Args& a, cudaStream_t stream) {
   const bool clamp = a.clip < 1.0f;
   if (a.symmetric) return clamp ? launch_t<FMT, true, true>(a, stream) : launch_t<FMT, true, false>(a, stream);
-  return clamp ? launch_t<FMT, false, true>(a, stream) : launch_t<FMT, false, false>(a, stream);
+  if constexpr (FMT == kFmtInt8Planes)   // the only asymmetric format
+    return clamp ? launch_t<FMT, false, true>(a, stream) : launch_t<FMT, false, false>(a, stream);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -237,8 +195,8 @@ cudaError_t launch_rotate_quant_8bit(const Rq8Args& a, cudaStream_t stream) {
   if (ep != cudaSuccess || handled) return ep;
   switch (a.format) {
     case kFmtInt8Planes: return launch_fmt<kFmtInt8Planes>(a, stream);
-    case kFmtE4M3: return a.symmetric ? launch_fmt<kFmtE4M3>(a, stream) : cudaErrorInvalidValue;
-    case kFmtInt4Bytes: return a.symmetric ? launch_fmt<kFmtInt4Bytes>(a, stream) : cudaErrorInvalidValue;
+    case kFmtE4M3: return launch_fmt<kFmtE4M3>(a, stream);
+    case kFmtInt4Bytes: return launch_fmt<kFmtInt4Bytes>(a, stream);
   }
   return cudaErrorNotSupported;
 }
