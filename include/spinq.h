@@ -375,15 +375,15 @@ spinq_status spinq_rope_rotate_quant_kv(const void* q_in, void* q_out, const voi
  *   lens     [B] int32 in [1, S] (device), or NULL for S everywhere.
  *   out      [B][Hq][D] fp16.
  *   workspace device buffer of spinq_decode_attention_workspace_bytes(B, S,
- *            Hq, Hkv, D) bytes, 16-byte aligned (the per-chunk partial
- *            results; no zeroing needed).
+ *            Hq, Hkv, D) bytes, 16-byte aligned (partial results
+ *            of long caches; no zeroing needed).
  *   Supported: D = 64 or 128, Hq / Hkv in {1, 2, 4, 8}, S * Hkv * D / 2 <
  *   2^31 (one batch's codes within 2 GiB).  Both products run
  *   on the tensor core with fp32 accumulation: q . u on the fp16 query and
  *   the exact codes, the value sum on the codes and fp16 weights
  *   p * v_scale / max(v_scale) (relative rounding 2^-11 per weight); the
- *   softmax and the scales in fp32.  Two kernels on `stream` (the chunks,
- *   then their merge).
+ *   softmax and the scales in fp32.  One kernel on `stream`, and a
+ *   second that merges partial results where the caches are long and few.
  */
 int64_t spinq_decode_attention_workspace_bytes(int64_t B, int64_t S, int64_t Hq, int64_t Hkv, int64_t D);
 spinq_status spinq_decode_attention_kv4(const void* q, const uint8_t* k_codes, const float* k_scale,

@@ -22,8 +22,9 @@
 // 2^8, so the fp16 weights p alpha' / r stay within [0, 256].
 // Split over the cache length (flash decoding):
 //
-//   partial kernel  grid (chunk, kv head, batch), 4 warps; a warp takes steps
-//     of 16 tokens.  Both products put the G query heads of the kv head on
+//   attention kernel  grid (chunk, kv head, batch), 4 warps; a sequence's own
+//     length is cut into equal chunks of whole steps; a warp takes steps of 16
+//     tokens.  Both products put the G query heads of the kv head on
 //     the MMA's N side (8 columns, columns >= G zero), so no accumulator
 //     register holds padding.  Scores S^T = K q^T: M = the 16 tokens,
 //     K = head_dim.  Lane (g, c) (g = lane / 4, c = lane % 4) loads bytes
@@ -35,9 +36,21 @@
 //     (one head, two tokens) by an 8x8 transpose (movmatrix), and lane (g, c)
 //     loads bytes [g D/16, (g+1) D/16) of value rows 2c, 2c+1, 2c+8, 2c+9,
 //     pairing two tokens' codes per fp16x2 register with a byte permute.
-//     Online softmax per step in base 2; the 4 warps merge at the end and
-//     write (max, sum, o[D]) of the chunk to the workspace.
-//   combine kernel  one warp per (batch, query head) merges the chunks.
+//     Online softmax per step in base 2; the 4 warps merge at the end.
+//     The chunks of a (batch, kv head) are the CTAs of one cluster, up to 8:
+//     each leaves (max, sum, o[G][D]) in its shared memory and after a cluster
+//     barrier the CTAs read each other's for their share of the output.  This
+//     replaces partial results in memory and a second kernel that merged them,
+//     whose warps waited on dependent loads (8 us alone for 9 chunks, 11 for
+//     32).  Both passes, graphs of calls on rotating caches, before -> now:
+//     8 sequences of 2048..4096 tokens 16.5 -> 13.0 us (28 MB, 4.2 us of HBM),
+//     16 of up to 1024 (48 / 12 heads, D 64) 11.3 -> 8.8, 77 of up to 512
+//     17.1 -> 14.4, 64 of up to 2048 37.2 -> 34.2, one of up to 2048 11.0 ->
+//     5.3 and of up to 8192 21.5 -> 8.9.  What is left is the issue rate (about
+//     250 instructions per warp and step, half of them unpacking) and, for
+//     short caches, the launch and one round trip to memory.
+//   combine kernel  where several clusters share a (batch, kv head): one warp
+//     per (batch, query head) merges the clusters' results.
 #include <cuda_fp16.h>
 #include <float.h>
 
@@ -50,6 +63,7 @@ namespace {
 
 constexpr int kAttnWarps = 4;
 constexpr int kAttnCtasPerSm = 4;   // resident CTAs per SM the chunking plans for
+constexpr int kAttnMaxCluster = 8;
 constexpr int kAttnStages = 4;      // 16-token stages in each warp's copy ring
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -111,9 +125,36 @@ __device__ __forceinline__ int stage_idx(int h, int d) {
   return h * (D + D / 16 + 4) + d + d / 16;
 }
 
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
+// Barrier of all threads of the cluster that does not ask for converged warps.
+__device__ __forceinline__ void cluster_sync_threads() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+
+// Shared memory of a CTA: the warps' rings, then the warps' (max, sum) and
+// their weights in the merge, then the CTA's merged (max, sum) and output.
 template <int D, int G>
-__global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_kernel(AttnArgs a, int chunk_len,
-                                                                                       int nchunk) {
+struct AttnSmem {
+  static constexpr int NW = kAttnWarps;
+  static constexpr int RING = NW * AttnRing<D>::WARP;
+  static constexpr int ML = RING, F = ML + 2 * NW * G * 4, CML = F + NW * G * 4, O = CML + 2 * G * 4;
+  static constexpr int TOTAL = O + G * D * 4;
+  static_assert(O % 8 == 0, "the merged output is read as pairs");
+};
+
+template <int D, int G>
+__global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(AttnArgs a, int nchunk, int C) {
+  constexpr int NW = kAttnWarps;
   constexpr int KW = D / 32;   // words of key codes per lane and token row (D/8 bytes)
   constexpr int VW = D / 64;   // words of value codes per lane and token row (D/16 bytes)
   constexpr int NS = D / 16;   // k16 slices of the score product
@@ -123,8 +164,15 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
   using Ring = AttnRing<D>;
   static_assert(G >= 1 && G <= 8, "at most 8 query heads per kv head");
   static_assert(G * (D + D / 16 + 4) * 4 <= Ring::WARP, "output staging fits in the warp's ring");
-  __shared__ __align__(16) unsigned char ring_s[kAttnWarps][Ring::WARP];
-  __shared__ float m_s[kAttnWarps][G], l_s[kAttnWarps][G];
+  using Smem = AttnSmem<D, G>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char(*ring_s)[Ring::WARP] = reinterpret_cast<unsigned char(*)[Ring::WARP]>(smem);
+  float(*m_s)[G] = reinterpret_cast<float(*)[G]>(smem + Smem::ML);
+  float(*l_s)[G] = m_s + NW;
+  float(*f_s)[G] = reinterpret_cast<float(*)[G]>(smem + Smem::F);
+  float* cm_s = reinterpret_cast<float*>(smem + Smem::CML);
+  float* cl_s = cm_s + G;
+  float* co_s = reinterpret_cast<float*>(smem + Smem::O);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, c = lane & 3;
   const int chunk = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
@@ -132,12 +180,14 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
   pdl_trigger();
   int64_t L = a.lens ? (int64_t)a.lens[b] : a.S;
   L = L < 0 ? 0 : (L > a.S ? a.S : L);
+  // the batch's own length in equal chunks of whole steps
+  const int64_t chunk_len = (int64_t)(((uint32_t)L + (uint32_t)nchunk - 1) / (uint32_t)nchunk + 15) / 16 * 16;
   const int64_t t0 = (int64_t)chunk * chunk_len;
   const int64_t t1 = t0 + chunk_len < L ? t0 + chunk_len : L;
   const int span = t1 > t0 ? (int)(t1 - t0) : 0;   // tokens of the chunk
   // this warp's steps: 16 tokens each, steps warp, warp + 4, ... of the chunk
   const int nstep_chunk = (span + 15) / 16;
-  const int nstep = nstep_chunk > warp ? (nstep_chunk - warp + kAttnWarps - 1) / kAttnWarps : 0;
+  const int nstep = nstep_chunk > warp ? (nstep_chunk - warp + NW - 1) / NW : 0;
 
   // Copy sources.  A step's rows past the chunk are still copied (their
   // scores are masked and their value scales zeroed below), clamped to the
@@ -159,7 +209,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
   // 64 scales
   auto issue = [&](int i) {
     if (i < nstep) {
-      const int tb = 16 * (warp + kAttnWarps * i);   // first token of the step, from t0
+      const int tb = 16 * (warp + NW * i);   // first token of the step, from t0
       const uint32_t st = ring + (uint32_t)(i % kAttnStages) * Ring::STAGE;
       if (tb + 15 <= last) {   // the whole step inside the cache
 #pragma unroll
@@ -197,7 +247,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
   // copies in flight
   float r = 0.f;
   for (int j = lane; j < 16 * nstep; j += 32) {
-    const int t = 16 * (warp + kAttnWarps * (j >> 4)) + (j & 15);
+    const int t = 16 * (warp + NW * (j >> 4)) + (j & 15);
     if (t < span) r = fmaxf(r, __ldg(a.v_scale + tok0 + (size_t)t * a.Hkv));
   }
 #pragma unroll
@@ -264,7 +314,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
     for (int u = 0; u < 2; ++u) {
       const int i = 2 * jp + u;
       st[u] = ring_s[warp] + (i % kAttnStages) * Ring::STAGE;
-      rem[u] = span - 16 * (warp + kAttnWarps * i);
+      rem[u] = span - 16 * (warp + NW * i);
     }
     // ---- scores S^T of both steps (two independent MMA chains)
     uint32_t kx[2][2][KW];
@@ -423,26 +473,89 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_partial_
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < G * (D + 2); e += kAttnWarps * 32) {
-    const int h = e / (D + 2), d = e % (D + 2);
-    float M = -FLT_MAX;
+  if (threadIdx.x < G) {
+    const int h = threadIdx.x;
+    float M = -FLT_MAX, den = 0.f;
 #pragma unroll
-    for (int w = 0; w < kAttnWarps; ++w) M = fmaxf(M, m_s[w][h]);
-    float val = 0.f;
-    if (d == 0) {
-      val = M;
-    } else {
+    for (int w = 0; w < NW; ++w) M = fmaxf(M, m_s[w][h]);
 #pragma unroll
-      for (int w = 0; w < kAttnWarps; ++w) {
-        const float fw = l_s[w][h] > 0.f ? exp2_approx(m_s[w][h] - M) : 0.f;
-        val += fw * (d == 1 ? l_s[w][h] : reinterpret_cast<const float*>(ring_s[w])[stage_idx<D>(h, d - 2)]);
-      }
+    for (int w = 0; w < NW; ++w) {
+      const float fw = l_s[w][h] > 0.f ? exp2_approx(m_s[w][h] - M) : 0.f;
+      den = fmaf(fw, l_s[w][h], den);
+      f_s[w][h] = fw;
     }
-    const size_t hq = (size_t)hk * G + h;
-    a.workspace[(((size_t)b * a.Hq + hq) * nchunk + chunk) * (D + 2) + d] = val;
+    cm_s[h] = M;
+    cl_s[h] = den;
+  }
+  __syncthreads();
+  // One pair of output elements (heads h, dims d, d + 1): the output itself
+  // where one cluster covers the cache, else the cluster's partial result
+  const int ncl = nchunk / C, cl = chunk / C;
+  auto finish = [&](int h, int d, float2 v, float M, float den) {
+    const size_t bh = (size_t)b * a.Hq + (size_t)hk * G + h;
+    if (ncl == 1) {
+      const float inv = den > 0.f ? 1.f / den : 0.f;
+      *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(a.out) + bh * D + d) =
+          __floats2half2_rn(v.x * inv, v.y * inv);
+    } else {
+      float* ws = a.workspace + (bh * ncl + cl) * (D + 2);
+      *reinterpret_cast<float2*>(ws + 2 + d) = v;
+      if (d == 0) *reinterpret_cast<float2*>(ws) = make_float2(M, den);
+    }
+  };
+  for (int e = threadIdx.x; e < G * D / 2; e += NW * 32) {
+    const int h = e / (D / 2), d = 2 * (e % (D / 2));
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      const float* ow = reinterpret_cast<const float*>(ring_s[w]) + stage_idx<D>(h, d);
+      v.x = fmaf(f_s[w][h], ow[0], v.x);
+      v.y = fmaf(f_s[w][h], ow[1], v.y);
+    }
+    if (C == 1)
+      finish(h, d, v, cm_s[h], cl_s[h]);
+    else
+      *reinterpret_cast<float2*>(co_s + 2 * e) = v;
+  }
+  if (C > 1) {
+    // the cluster's CTAs share the pairs; each reads every CTA's part
+    const int rank = chunk % C;
+    __syncwarp();
+    cluster_sync_threads();
+    for (int e = threadIdx.x + rank * (NW * 32); e < G * D / 2; e += C * (NW * 32)) {
+      const int h = e / (D / 2), d = 2 * (e % (D / 2));
+      const uint32_t om = smem_u32(co_s + 2 * e), mm = smem_u32(cm_s + h);
+      float mc[kAttnMaxCluster], lc[kAttnMaxCluster];
+      float2 oc[kAttnMaxCluster];
+      float M = -FLT_MAX, den = 0.f;
+#pragma unroll
+      for (int r2 = 0; r2 < kAttnMaxCluster; ++r2) {
+        mc[r2] = -FLT_MAX, lc[r2] = 0.f, oc[r2] = make_float2(0.f, 0.f);
+        if (r2 < C) {
+          const uint32_t m2 = mapa_shared(mm, (uint32_t)r2);
+          mc[r2] = ld_cluster_f32(m2);
+          lc[r2] = ld_cluster_f32(m2 + 4 * G);
+          oc[r2] = ld_cluster_f32x2(mapa_shared(om, (uint32_t)r2));
+        }
+      }
+#pragma unroll
+      for (int r2 = 0; r2 < kAttnMaxCluster; ++r2) M = fmaxf(M, mc[r2]);
+      float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int r2 = 0; r2 < kAttnMaxCluster; ++r2) {
+        const float f = lc[r2] > 0.f ? exp2_approx(mc[r2] - M) : 0.f;
+        den = fmaf(f, lc[r2], den);
+        v.x = fmaf(f, oc[r2].x, v.x);
+        v.y = fmaf(f, oc[r2].y, v.y);
+      }
+      finish(h, d, v, M, den);
+    }
+    __syncwarp();
+    cluster_sync_threads();   // no CTA leaves while another reads its part
   }
 }
 
+// nchunk: the clusters of a (batch, kv head)
 template <int D>
 __global__ void __launch_bounds__(128) attn_combine_kernel(AttnArgs a, int nchunk) {
   constexpr int DPL = D / 32;
@@ -488,25 +601,52 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(AttnArgs a, int nchun
   for (int i = 0; i < DPL; i += 2) *reinterpret_cast<__half2*>(out + i) = __floats2half2_rn(o[i] * inv, o[i + 1] * inv);
 }
 
+// CTAs per cluster and clusters per (batch, kv head).  Up to 8 chunks are one
+// cluster and one kernel.  Where the SMs would take more (few sequences), one
+// cluster of 8 stays ahead of several and their merge up to about 1024 tokens
+// per chunk: 32 query and 8 kv heads, D 128, lengths S / 2 to S, us,
+//                              1 x 8   2 x 8   4 x 8   8 x 8
+//   1 sequence,  S =  2048      5.25    7.2
+//   1 sequence,  S =  8192      8.9    10.2     9.5    10.3
+//   2 sequences, S = 16384     16.9    14.4    15.7
+//   1 sequence,  S = 32768     22.5             17.0    16.2
+struct AttnPlan {
+  int cluster, clusters;
+};
+
+AttnPlan plan_attention(int64_t B, int64_t S, int64_t Hkv) {
+  const int n = decode_attention_chunks(B, S, Hkv);
+  if (n <= kAttnMaxCluster) return {n, 1};
+  const int64_t by_len = (S + 1024 * kAttnMaxCluster - 1) / (1024 * kAttnMaxCluster);
+  return {kAttnMaxCluster, (int)(by_len < n / kAttnMaxCluster ? by_len : n / kAttnMaxCluster)};
+}
+
 template <int D, int G>
-cudaError_t launch_dg(const AttnArgs& a, int nchunk, cudaStream_t stream) {
-  const int chunk_len = (int)((a.S + nchunk - 1) / nchunk);
-  cudaError_t e = launch_pdl(attn_partial_kernel<D, G>, dim3((unsigned)nchunk, (unsigned)a.Hkv, (unsigned)a.B),
-                             dim3(kAttnWarps * 32), 0, stream, 1, a, chunk_len, nchunk);
+cudaError_t launch_dg(const AttnArgs& a, cudaStream_t stream) {
+  const AttnPlan p = plan_attention(a.B, a.S, a.Hkv);
+  const int nchunk = p.cluster * p.clusters;
+  const size_t smem = AttnSmem<D, G>::TOTAL;
+  int per_sm = 0;
+  cudaError_t e = prepare_launch(attn_kernel<D, G>, kAttnWarps * 32, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  const int64_t groups = (a.B * a.Hq + 3) / 4;
-  e = launch_pdl(attn_combine_kernel<D>, dim3((unsigned)groups), dim3(128), 0, stream, 1, a, nchunk);
+  e = launch_pdl(attn_kernel<D, G>, dim3((unsigned)nchunk, (unsigned)a.Hkv, (unsigned)a.B), dim3(kAttnWarps * 32),
+                 smem, stream, p.cluster, a, nchunk, p.cluster);
   if (e != cudaSuccess) return e;
+  if (p.clusters > 1) {
+    const int64_t groups = (a.B * a.Hq + 3) / 4;
+    e = launch_pdl(attn_combine_kernel<D>, dim3((unsigned)groups), dim3(128), 0, stream, 1, a, p.clusters);
+    if (e != cudaSuccess) return e;
+  }
   return cudaGetLastError();
 }
 
 template <int D>
-cudaError_t launch_d(const AttnArgs& a, int nchunk, cudaStream_t stream) {
+cudaError_t launch_d(const AttnArgs& a, cudaStream_t stream) {
   switch (a.Hq / a.Hkv) {
-    case 1: return launch_dg<D, 1>(a, nchunk, stream);
-    case 2: return launch_dg<D, 2>(a, nchunk, stream);
-    case 4: return launch_dg<D, 4>(a, nchunk, stream);
-    case 8: return launch_dg<D, 8>(a, nchunk, stream);
+    case 1: return launch_dg<D, 1>(a, stream);
+    case 2: return launch_dg<D, 2>(a, stream);
+    case 4: return launch_dg<D, 4>(a, stream);
+    case 8: return launch_dg<D, 8>(a, stream);
   }
   return cudaErrorNotSupported;
 }
@@ -524,9 +664,9 @@ int decode_attention_chunks(int64_t B, int64_t S, int64_t Hkv) {
   return (int)(n < 1 ? 1 : n);
 }
 
-cudaError_t launch_decode_attention(const AttnArgs& a, int nchunk, cudaStream_t stream) {
-  if (a.D == 128) return launch_d<128>(a, nchunk, stream);
-  if (a.D == 64) return launch_d<64>(a, nchunk, stream);
+cudaError_t launch_decode_attention(const AttnArgs& a, cudaStream_t stream) {
+  if (a.D == 128) return launch_d<128>(a, stream);
+  if (a.D == 64) return launch_d<64>(a, stream);
   return cudaErrorNotSupported;
 }
 

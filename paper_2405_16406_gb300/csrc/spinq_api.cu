@@ -408,7 +408,7 @@ spinq_status spinq_decode_attention_kv4(const void* q, const uint8_t* k_codes, c
   if (B == 0) return SPINQ_OK;
   AttnArgs a{q, k_codes, k_scale, k_zero, v_codes, v_scale, v_zero, lens, B, S, Hq, Hkv, (int)D, softmax_scale,
              out, static_cast<float*>(workspace)};
-  return from_cuda(launch_decode_attention(a, decode_attention_chunks(B, S, Hkv), static_cast<cudaStream_t>(stream)));
+  return from_cuda(launch_decode_attention(a, static_cast<cudaStream_t>(stream)));
 }
 
 spinq_status spinq_debug_set_wait_limit_ns(int64_t ns) {

@@ -99,10 +99,10 @@ struct AttnArgs {
   float* workspace;
 };
 
-// Chunks of the cache length that the decode attention splits over (the
-// workspace holds B * Hq * chunks * (D + 2) floats).
+// Most chunks of the cache length that the decode attention splits over (the
+// workspace is B * Hq * chunks * (D + 2) floats; the launch takes fewer).
 int decode_attention_chunks(int64_t B, int64_t S, int64_t Hkv);
-cudaError_t launch_decode_attention(const AttnArgs& a, int chunks, cudaStream_t stream);
+cudaError_t launch_decode_attention(const AttnArgs& a, cudaStream_t stream);
 
 struct GemmArgs {
   const uint8_t* a_codes;
