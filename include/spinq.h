@@ -175,7 +175,10 @@ int64_t spinq_w4a4_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K);
  * disjoint part of the weights; the slices' exact integer partial
  * accumulators are summed in `workspace` and the last slice of each
  * 128-channel tile applies the epilogue (with a single slice the CTA writes
- * the outputs itself and no workspace is used).  For M > 256 the call runs
+ * the outputs itself and no workspace is used).  Under the automatic choice
+ * (no kernel and no number of slices selected) most calls of up to 128 tokens
+ * instead take clusters of up to 8 CTAs per 128 channels that sum their slices
+ * over distributed shared memory; `workspace` is then checked but not touched.  For M > 256 the call runs
  * the same kernel as spinq_w4a4_gemm and does not touch `workspace`.
  *   workspace       device buffer of spinq_w4a4_gemm_workspace_bytes(M, N, K)
  *                   bytes, 16-byte aligned, all zero before the first call;
@@ -330,7 +333,9 @@ int spinq_w4a4_gemm_plan(int64_t M, int64_t N, int64_t K);
 /*
  * spinq_w4a4_gemm_splitk_plan -- the kernel that spinq_w4a4_gemm_splitk runs
  * for an M x N x K call given a workspace of spinq_w4a4_gemm_workspace_bytes
- * bytes: SPINQ_GEMM_SPLITK, with *nsplit (may be NULL) set to its number of K
+ * bytes, before the choice of clusters described there (which needs none and
+ * keeps this answer, so that workspaces sized by it stay valid):
+ * SPINQ_GEMM_SPLITK, with *nsplit (may be NULL) set to its number of K
  * slices per 128-channel tile (1: no slicing, no workspace), or the kernel
  * spinq_w4a4_gemm would run (*nsplit = 0).  -1 for shapes the call rejects.
  * Launches nothing.

@@ -415,7 +415,7 @@ spinq_status spinq_debug_set_wait_limit_ns(int64_t ns) {
   if (ns <= 0) return SPINQ_EINVAL;
   const uint64_t v = (uint64_t)ns;
   if (set_wait_limit_paley(v) != cudaSuccess || set_wait_limit_gemm(v) != cudaSuccess ||
-      set_wait_limit_fp8(v) != cudaSuccess)
+      set_wait_limit_fp8(v) != cudaSuccess || set_wait_limit_decode_cluster(v) != cudaSuccess)
     return SPINQ_ECUDA;
   return SPINQ_OK;
 }

@@ -165,6 +165,16 @@ bool w4a4_gemv_tc_streamed(int64_t K);
 cudaError_t launch_w4a4_gemm_splitk(const GemmArgs& a, void* workspace, int64_t workspace_bytes,
                                     cudaStream_t stream);
 
+// Decode GEMM for M <= kDecodeClusterMaxM tokens whose K range is split over a cluster of
+// `cluster` CTAs (w4a4_decode_cluster.cu; 1..kDecodeMaxCluster, at most
+// K / 128), no workspace.
+constexpr int kDecodeMaxCluster = 8;
+constexpr int64_t kDecodeClusterMaxM = 128;
+cudaError_t launch_w4a4_decode_cluster(const GemmArgs& a, int cluster, cudaStream_t stream);
+// Clusters of that many CTAs that can be resident at once (0 if none).
+int w4a4_decode_clusters(int cluster);
+cudaError_t set_wait_limit_decode_cluster(uint64_t ns);
+
 struct CayleyArgs {
   const float* R;     // [batch][n][n]
   const float* grad;  // [batch][n][n] loss gradient

@@ -1283,6 +1283,7 @@ namespace {
 struct DecodePlan {
   bool prefill;
   int nsplit;
+  double us;
 };
 
 DecodePlan plan_decode(int64_t M, int64_t N, int64_t K, int ns_lo, int ns_hi, bool allow_prefill) {
@@ -1303,8 +1304,11 @@ DecodePlan plan_decode(int64_t M, int64_t N, int64_t K, int ns_lo, int ns_hi, bo
       best_ns = ns;
     }
   }
-  if (allow_prefill && choose_prefill(M, N, K, true).us + 3.0 < best) return {true, 0};
-  return {false, best_ns};
+  if (allow_prefill) {
+    const double pre = choose_prefill(M, N, K, true).us + 3.0;
+    if (pre < best) return {true, 0, pre};
+  }
+  return {false, best_ns, best};
 }
 
 constexpr int kMaxSplit = 64;
@@ -1321,6 +1325,44 @@ DecodePlan plan_splitk_entry(int64_t M, int64_t N, int64_t K, bool room) {
   if (!room) lo = hi = 1;
   // a forced split-K kernel runs whatever the model predicts for the others
   return plan_decode(M, N, K, lo, hi, g_gemm_kernel.load(std::memory_order_relaxed) != SPINQ_GEMM_SPLITK);
+}
+
+// Cluster size with which the clustered kernel (w4a4_decode_cluster.cu) takes
+// a call of up to 128 tokens under the automatic choice, 0 where the plan's
+// route (`other_us`) is predicted to be as fast.  Microseconds, fitted on GB300
+// over K x N in {2048, 3072, 4096, 8192, 14336} x {2048 .. 16384}, 9 to 128
+// tokens and clusters of 1 to 6:
+//   waves (4.3 + 0.021 M + steps (0.27 + 0.0018 MN)),
+// steps the 128-deep K steps of a CTA.  Measured with the activation quantizer
+// before it (graphs over rotating weights), the plan's route -> this one:
+//   24 tokens:  4096 -> 4096 11.6 -> 9.3 us, 14336 -> 4096 18.8 -> 17.6
+//   77 tokens:  4096 -> 4096 22.5 -> 11.7, 4096 -> 6144 23.5 -> 14.9,
+//               14336 -> 4096 36.3 -> 21.5, 3072 -> 16384 21.1 -> 19.3
+//   128 tokens: 8192 -> 3072 30.0 -> 17.7
+// and the plan's route stays ahead where the tiles need a second wave (4096 ->
+// 28672 at 77 tokens, 128-row tiles: 26.4 against 33.8) and for wide outputs
+// at 128 tokens (3072 -> 16384: 21.9 against 23.0).  It has to win by half a
+// microsecond: below that lie calls of a few K steps, where start-up is all
+// there is (24 tokens, 256 -> 512: 5.8 against 6.4).
+int decode_cluster(int64_t M, int64_t N, int64_t K, double other_us) {
+  if (M > kDecodeClusterMaxM || g_gemm_kernel.load(std::memory_order_relaxed) != SPINQ_GEMM_AUTO ||
+      g_split_k.load(std::memory_order_relaxed) != 0)
+    return 0;
+  const int64_t tiles = (N + 127) / 128, ks = K / 128;
+  const double step = 0.27 + 0.0018 * (double)((M + 15) / 16 * 16);
+  int best = 0;
+  other_us -= 0.5;
+  for (int c = 1; c <= kDecodeMaxCluster && c <= ks; ++c) {
+    const int64_t resident = w4a4_decode_clusters(c);
+    if (resident < 1) continue;
+    const double us = (double)((tiles + resident - 1) / resident) *
+                      (4.3 + 0.021 * (double)M + (double)((ks + c - 1) / c) * step);
+    if (us < other_us) {
+      other_us = us;
+      best = c;
+    }
+  }
+  return best;
 }
 
 bool gemv_serves(int64_t M, int64_t K) {
@@ -1364,6 +1406,7 @@ cudaError_t launch_w4a4_gemm_splitk(const GemmArgs& a, void* workspace, int64_t 
   }
   const bool room = workspace != nullptr && workspace_bytes >= split_workspace_bytes(a.M, a.N);
   const DecodePlan p = plan_splitk_entry(a.M, a.N, a.K, room);
+  if (const int c = decode_cluster(a.M, a.N, a.K, p.us)) return launch_w4a4_decode_cluster(a, c, stream);
   if (p.prefill) return launch_w4a4_gemm(a, stream);
   float* ws_acc = p.nsplit > 1 ? static_cast<float*>(workspace) : nullptr;
   int* ws_cnt = ws_acc == nullptr ? nullptr : reinterpret_cast<int*>(static_cast<char*>(workspace) + a.M * a.N * 4);
