@@ -837,11 +837,11 @@ def attention_records(dev, hbm_peak):
     return {
         "f2_rope_r3_kv4_B8_S4096": {"us": round(rope_us, 2), "bytes": rope_bytes,
                                      "frac_hbm": round(rope_bytes / rope_us / 1e3 / hbm_peak, 4),
-                                     "kernel": "rotate_quant_kv_kernel with the RoPE stage"},
+                                     "kernel": "rope_rotate_quant_kv_kernel"},
         "f2_decode_attention_kv4_B8_S4096_Hq32_Hkv8_D128": {
             "us": round(att_us, 2), "bytes": att_bytes, "frac_hbm": round(att_bytes / att_us / 1e3 / hbm_peak, 4),
-            "chunks": int(ws.numel() // (B * Hq * (Dd + 2) * 4)),
-            "kernel": "attn_partial_kernel + attn_combine_kernel",
+            "workspace_chunks": int(ws.numel() // (B * Hq * (Dd + 2) * 4)),
+            "kernel": "attn_kernel",
             "checked": "batch 0's 32 heads vs the oracle on the same codes"}}
 
 
