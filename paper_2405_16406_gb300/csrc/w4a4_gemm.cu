@@ -16,8 +16,8 @@
 // (sum_k u_w = rowsum_n + 8 K cancels the 64 K term).  sum_k u_a is counted
 // by the unpack warps while they expand the activation tiles.
 //
-// Persistent kernel: one CTA per SM walks the output tiles (128 x 256 or
-// 256 x 256, M fastest so that concurrently running CTAs share weight tiles
+// Persistent kernel: one CTA per SM walks the output tiles (128 x 256,
+// 256 x 256 or 256 x 192, M fastest so that concurrently running CTAs share weight tiles
 // in L2).  Warp
 // roles (704 threads):
 //   warp 0       TMA producer: packed A [128 x 64 B] and B [256 x 64 B] tiles
@@ -144,7 +144,6 @@ struct Cfg {
   static constexpr int NP = MT == 1 ? 3 : 2;   // packed (TMA) stages
   static constexpr int NU = MT == 1 ? 3 : 2;   // unpacked (MMA operand) stages
   static constexpr int TA = BMT * 4 / (kUnpackWarps * 32);   // A chunks per unpack thread
-  static constexpr int TB = BN * 4 / (kUnpackWarps * 32);    // B chunks per unpack thread
   static constexpr uint32_t uA = 0;
   static constexpr uint32_t uB = uA + NU * BMT * 128;
   static constexpr uint32_t pA = uB + NU * BN * 128;
@@ -191,12 +190,12 @@ struct Cfg {
 //   evaluated as y = s_n * fma(alpha * 2^18, acc, c + d * rw_n) with
 //   c = -8 alpha rs_a and d = beta' - 8 alpha (the roundings of the other
 //   kernels, so that every kernel gives the same bits).
-template <bool ASYM, bool ACC_OUT>
+template <int TN, bool ASYM, bool ACC_OUT>
 __device__ __forceinline__ void epi256_share(const GemmArgs& args, uint32_t tq, int q, int lane, int part,
                                              int nparts, int64_t m_tile0, int64_t n0, const float* col_s,
                                              const float* col_r, int rsa0, int rsa1, uint32_t stage,
                                              uint64_t* acc_empty, uint64_t* stg_free) {
-  constexpr int NBLK = 2 * (BN / 64);
+  constexpr int NBLK = 2 * (TN / 64);
   // per-row constants of the two accumulators, kept in scalars: the block
   // loop selects them with a runtime accumulator index
   F2 as2_0, cm2_0, dm2_0, as2_1, cm2_1, dm2_1;
@@ -217,7 +216,7 @@ __device__ __forceinline__ void epi256_share(const GemmArgs& args, uint32_t tq, 
   const uint32_t srow = stage + (uint32_t)lane * 128;
 #pragma unroll 1
   for (int g = part; g < NBLK; g += nparts) {
-    const int mt = g / (BN / 64), cb = g % (BN / 64);
+    const int mt = g / (TN / 64), cb = g % (TN / 64);
     const int64_t m = mt ? m_1 : m_0;
     const F2 as2 = mt ? as2_1 : as2_0, cm2 = mt ? cm2_1 : cm2_0, dm2 = mt ? dm2_1 : dm2_0;
     const int rsam = mt ? rsa1 : rsa0;
@@ -308,7 +307,7 @@ __device__ __forceinline__ void epi256_share(const GemmArgs& args, uint32_t tq, 
 // sums and the column constants of that tile, then runs its share.  False
 // when a wait gave up (the share is skipped; the accumulator and staging
 // barriers are then left to the bounded waits of the other roles).
-template <bool ASYM, bool ACC_OUT>
+template <int TN, bool ASYM, bool ACC_OUT>
 __device__ __forceinline__ bool unpack_epi_share(const GemmArgs& args, uint32_t tmem, int warp, int lane, int plt,
                                                  int ptile, int m_tiles, uint64_t* acc_full, uint64_t* acc_empty,
                                                  uint64_t* rs_full, uint64_t* cols_full, uint64_t* stg_free,
@@ -328,17 +327,20 @@ __device__ __forceinline__ bool unpack_epi_share(const GemmArgs& args, uint32_t 
   const int rsa1 = rs_a[(rb * kUnpackGroups) * BMT + r1] + rs_a[(rb * kUnpackGroups + 1) * BMT + r1];
   const float* col_s = cols + rb * 2 * BN;
   constexpr int NPARTS = Cfg<2>::EPI_PARTS;
-  epi256_share<ASYM, ACC_OUT>(args, tmem + ((uint32_t)(q * 32) << 16), q, lane, part, NPARTS,
-                              (int64_t)(ptile % m_tiles) * BMT, (int64_t)(ptile / m_tiles) * BN, col_s, col_s + BN,
-                              rsa0, rsa1, stage, &acc_empty[0], stg_free);
+  epi256_share<TN, ASYM, ACC_OUT>(args, tmem + ((uint32_t)(q * 32) << 16), q, lane, part, NPARTS,
+                              (int64_t)(ptile % m_tiles) * BMT, (int64_t)(ptile / m_tiles) * TN, col_s,
+                              col_s + BN, rsa0, rsa1, stage, &acc_empty[0], stg_free);
   return true;
 }
 
-template <int MT, bool ASYM, bool ACC_OUT>
+// TN: columns of a tile, up to BN, which the stages are laid out for.
+template <int MT, bool ASYM, bool ACC_OUT, int TN>
 __global__ void __launch_bounds__(kThreads, 1)
     w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      GemmArgs args, int num_k, int m_tiles, int num_tiles) {
   using L = Cfg<MT>;
+  constexpr int bn = TN, TB = TN * 4 / (kUnpackWarps * 32);   // B chunks per unpack thread
+  static_assert(TN % 64 == 0 && TN <= BN, "whole chunks per unpack thread, whole epilogue blocks");
   constexpr int BMT = L::BMT, NP = L::NP, NU = L::NU, NACC = L::NACC;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-aligned base derived from the shared array itself, so that the
@@ -391,7 +393,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     prefetch_tmap(&tmB);
     if ((int)blockIdx.x < num_tiles)
       for (int kt = 0; kt < kPrefetchSteps && kt < num_k; ++kt)
-        tma_prefetch_2d(&tmB, kt * 64, (int)(blockIdx.x / m_tiles) * BN);
+        tma_prefetch_2d(&tmB, kt * 64, (int)(blockIdx.x / m_tiles) * bn);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, 512);
@@ -411,14 +413,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       int& it = prod_it;
       bool stop = args.debug_stall != 0;   // a test of the time-outs issues no copies
       for (int tile = blockIdx.x; tile < num_tiles && !stop; tile += gridDim.x) {
-        const int32_t m0 = (tile % m_tiles) * BMT, n0 = (tile / m_tiles) * BN;
+        const int32_t m0 = (tile % m_tiles) * BMT, n0 = (tile / m_tiles) * bn;
         for (int kt = 0; kt < num_k; ++kt, ++it) {
           const int s = it % NP;
           if (!wait_or_abort(&empty_p[s], ((it / NP) & 1) ^ 1, abort_flag, 1)) {
             stop = true;
             break;
           }
-          mbar_arrive_expect_tx(&full_p[s], (BMT + BN) * 64);
+          mbar_arrive_expect_tx(&full_p[s], (uint32_t)(BMT + bn) * 64);
           tma_load_2d(base + L::pA + s * BMT * 64, &tmA, &full_p[s], kt * 64, m0);
           tma_load_2d(base + L::pB + s * BN * 64, &tmB, &full_p[s], kt * 64, n0);
         }
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_e4m3_f32(128, BN);
+      constexpr uint32_t idesc = umma_idesc_e4m3_f32(128, bn);
       int it = 0, lt = 0;
       bool stop = false;
       for (int tile = blockIdx.x; tile < num_tiles && !stop; tile += gridDim.x, ++lt) {
@@ -492,11 +494,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         return false;
       const uint32_t PA = sbase + L::pA + s * BMT * 64, PB = sbase + L::pB + s * BN * 64;
       const uint32_t UA = sbase + L::uA + su * BMT * 128, UB = sbase + L::uB + su * BN * 128;
-      uint4 wa[L::TA], wb[L::TB];
+      uint4 wa[L::TA], wb[TB];
 #pragma unroll
       for (int j = 0; j < L::TA; ++j) wa[j] = lds128(PA + l0 + 4096 * j);
 #pragma unroll
-      for (int j = 0; j < L::TB; ++j) wb[j] = lds128(PB + l0 + 4096 * j);
+      for (int j = 0; j < TB; ++j) wb[j] = lds128(PB + l0 + 4096 * j);
       // packed stage consumed, once every lane's loads have read it
       wait_loaded(wa, scratch);
       wait_loaded(wb, scratch);
@@ -511,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         sts128(UA + (s0 ^ 16u) + 8192 * j, hi);
       }
 #pragma unroll
-      for (int j = 0; j < L::TB; ++j) {
+      for (int j = 0; j < TB; ++j) {
         uint4 lo, hi;
         unpack16(wb[j], 0x88888888u, lo, hi);
         sts128(UB + s0 + 8192 * j, lo);
@@ -585,8 +587,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int h = warp - kFirstUnpackWarp;   // 0..15
         const uint32_t stage = sbase + (h < 8 ? L::uA + (1 - first) * BMT * 128 : L::uB + (1 - first) * BN * 128) +
                                (uint32_t)(h & 7) * L::EPI_STAGE;
-        if (!unpack_epi_share<ASYM, ACC_OUT>(args, tmem, warp, lane, lt, tile, m_tiles, acc_full, acc_empty, rs_full,
-                                             cols_full, stg_free, rs_a, cols, stage, abort_flag))
+        if (!unpack_epi_share<TN, ASYM, ACC_OUT>(args, tmem, warp, lane, lt, tile, m_tiles, acc_full, acc_empty,
+                                             rs_full, cols_full, stg_free, rs_a, cols, stage, abort_flag))
           break;
         if (1 - first == grp) stg_due = lt;
       }
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int lt = 0;
     for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x, ++lt) {
       const int b = lt % NACC, rb = lt & 1;
-      const int64_t n0 = (int64_t)(tile / m_tiles) * BN;
+      const int64_t n0 = (int64_t)(tile / m_tiles) * bn;
       const int64_t m_tile0 = (int64_t)(tile % m_tiles) * BMT;
       // column constants of this tile into the buffer of its parity.  Its
       // last readers worked on tile lt - 2: with 256-row tiles they all
@@ -632,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive(&rs_empty[rb]);
       const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * MT * BN);
       if constexpr (MT == 2) {
-        epi256_share<ASYM, ACC_OUT>(args, tq, q, lane, 0, L::EPI_PARTS, m_tile0, n0, col_s, col_r, rsa[0],
+        epi256_share<TN, ASYM, ACC_OUT>(args, tq, q, lane, 0, L::EPI_PARTS, m_tile0, n0, col_s, col_r, rsa[0],
                                     rsa[MT - 1], smem_u32(base + L::estage) + (uint32_t)(q * L::EPI_STAGE),
                                     &acc_empty[b], nullptr);
         continue;
@@ -1073,20 +1075,32 @@ bool encode_y_map(CUtensorMap* map, void* y, int64_t M, int64_t N) {
 
 namespace {
 
-template <int MT, bool ASYM, bool ACC_OUT>
-cudaError_t launch_t(const GemmArgs& a, cudaStream_t stream) {
+// Width of 256-row tiles: 192 columns where they save work for whole waves.
+// us per tile: 0.66 per 128-deep K step + 5 for the epilogue at 256 columns,
+// 0.60 + 4 at 192 (a K step is bound by the unpack warps, 512 rows against 448).
+// 1531 x 4096 -> 14336 81.7 us at 256, 72.3 at 192 (3 waves of either); 512 x
+// 4096 -> 4096 28.5 and 25.5 (one); 2048 x 14336 -> 4096 81.3 and 143 (one, two).
+int tile256_width(int64_t M, int64_t N, int64_t K, int64_t sms) {
+  const int64_t m_tiles = (M + 255) / 256, ks = K / 128;
+  const double wide = (double)((m_tiles * ((N + BN - 1) / BN) + sms - 1) / sms) * (0.66 * (double)ks + 5.0);
+  const double slim = (double)((m_tiles * ((N + 191) / 192) + sms - 1) / sms) * (0.60 * (double)ks + 4.0);
+  return slim < wide ? 192 : BN;
+}
+
+template <int MT, bool ASYM, bool ACC_OUT, int TN>
+cudaError_t launch_tn(const GemmArgs& a, cudaStream_t stream) {
   using L = Cfg<MT>;
   CUtensorMap tmA, tmB;
   if (!encode_packed_map(&tmA, a.a_codes, a.M, a.K, L::BMT)) return cudaErrorNotSupported;
-  if (!encode_packed_map(&tmB, a.w_codes, a.N, a.K, BN)) return cudaErrorNotSupported;
-  auto kern = w4a4_gemm_kernel<MT, ASYM, ACC_OUT>;
+  const int sms = device_sm_count();
+  if (!encode_packed_map(&tmB, a.w_codes, a.N, a.K, TN)) return cudaErrorNotSupported;
+  auto kern = w4a4_gemm_kernel<MT, ASYM, ACC_OUT, TN>;
   const size_t smem = L::dyn_bytes;
   int per_sm = 0;
   cudaError_t e = prepare_launch(kern, kThreads, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  const int sms = device_sm_count();
   const int m_tiles = (int)((a.M + L::BMT - 1) / L::BMT);
-  const int n_tiles = (int)((a.N + BN - 1) / BN);
+  const int n_tiles = (int)((a.N + TN - 1) / TN);
   const int tiles = m_tiles * n_tiles;
   const int grid = tiles < sms ? tiles : sms;
   GemmArgs la = a;
@@ -1095,6 +1109,15 @@ cudaError_t launch_t(const GemmArgs& a, cudaStream_t stream) {
                  tiles);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
+}
+
+template <int MT, bool ASYM, bool ACC_OUT>
+cudaError_t launch_t(const GemmArgs& a, cudaStream_t stream) {
+  if constexpr (MT == 2) {
+    if (tile256_width(a.M, a.N, a.K, device_sm_count()) == 192)
+      return launch_tn<MT, ASYM, ACC_OUT, 192>(a, stream);
+  }
+  return launch_tn<MT, ASYM, ACC_OUT, BN>(a, stream);
 }
 
 template <int MT>
