@@ -386,8 +386,9 @@ spinq_status spinq_rope_rotate_quant_kv(const void* q_in, void* q_out, const voi
  *   2^31 (one batch's codes within 2 GiB).  Both products run
  *   on the tensor core with fp32 accumulation: q . u on the fp16 query and
  *   the exact codes, the value sum on the codes and fp16 weights
- *   p * v_scale / max(v_scale) (relative rounding 2^-11 per weight); the
- *   softmax and the scales in fp32.  One kernel on `stream`, and a
+ *   p * v_scale / max(v_scale) (relative rounding 2^-11 per weight, of which
+ *   the part common to all codes is added back in fp32); the softmax and the
+ *   scales in fp32.  One kernel on `stream`, and a
  *   second that merges partial results where the caches are long and few.
  */
 int64_t spinq_decode_attention_workspace_bytes(int64_t B, int64_t S, int64_t Hq, int64_t Hkv, int64_t D);

@@ -12,8 +12,9 @@
 //   s_t = scale * (alpha_t (q . u_t) + beta_t sum_d q_d),
 // and the value sum is
 //   o = sum_t p_t (alpha'_t u'_t + beta'_t)
-//     = r * sum_t (p_t alpha'_t / r) u'_t + sum_t p_t beta'_t,
-// so both products take the raw codes u as fp16 operands of the tensor core
+//     = r * sum_t P'_t u'_t + sum_t (p_t (beta'_t + 8 alpha'_t) - 8 r P'_t),
+// P'_t = p_t alpha'_t / r rounded to fp16 (its rounding meets u' - 8), so both
+// products take the raw codes u as fp16 operands of the tensor core
 // (mma.sync m16n8k16, fp32 accumulation).  A code is unpacked by one mask:
 // read as an fp16 bit pattern it is the subnormal u 2^-24 (or 16 u 2^-24),
 // which the tensor core multiplies exactly, and the product with an fp16
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(A
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, off));
-  const float rinv = r > 0.f ? 1.f / r : 0.f;
+  const float rinv = r > 0.f ? 1.f / r : 0.f, m8r = -8.f * r;
 
   // B fragments of query head g (zero for g >= G) in the order the key codes
   // meet the MMA: slice 2w + e, k = 2c, 2c+1 take dimensions 2(cD/8 + 4w + e)
@@ -292,8 +293,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(A
 
   // Running state of heads 2c + e in this lane: the score maximum m (base 2),
   // the lane's share (tokens g, g + 8 of each step) of the weight sum l and of
-  // sum p beta', and o[mu] = sum p alpha' u / r for dimensions gD/8 + 2mu
-  // (o[mu][e]) and gD/8 + 2mu + 1 (o[mu][2 + e]).
+  // sum p (beta' + 8 alpha') - 8 r P', and o[mu] = sum P' u for dimensions
+  // gD/8 + 2mu (o[mu][e]) and gD/8 + 2mu + 1 (o[mu][2 + e]).
   float o[NM][4];
 #pragma unroll
   for (int mu = 0; mu < NM; ++mu) o[mu][0] = o[mu][1] = o[mu][2] = o[mu][3] = 0.f;
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(A
         const bool in = g + 8 * hf < rem[u];
         const float ka = (ks * kCodeScale) * f.x;
         wv[u][hf] = in ? f.z * rinv : 0.f;
-        zv[u][hf] = in ? f.w : 0.f;
+        zv[u][hf] = in ? fmaf(8.f, f.z, f.w) : 0.f;   // beta' + 8 alpha'
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           sc[u][hf][e] = in ? fmaf(ka, sacc[u][2 * hf + e], f.y * qsk[e]) : -FLT_MAX;
@@ -379,25 +380,42 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(A
     // (base 2), so the weights p stay below 2^8 and the accumulators are
     // rescaled rarely.  The pair's first step holds a token of the chunk, so
     // m is finite from the first pair on and the masked scores give p = 0.
-    float p[2][2][2], corr[2];
+    float corr[2], mnew[2];
     bool moved = false;
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const float mnew = mx[e] > m[e] + 8.f ? mx[e] : m[e];
-      moved |= mnew != m[e];
-      corr[e] = exp2_approx(m[e] - mnew);
-      float ps = 0.f, pz = 0.f;
+      mnew[e] = mx[e] > m[e] + 8.f ? mx[e] : m[e];
+      moved |= mnew[e] != m[e];
+      corr[e] = exp2_approx(m[e] - mnew[e]);
+      m[e] = mnew[e];
+    }
+    // P' = p alpha' / r in fp16 for the value product.  Its rounding would meet
+    // the codes u in 0 .. 15, whose mean is far from zero; the sum beside the
+    // product takes 8 (p alpha' - P' r) on top of p beta', so that what the
+    // rounding meets in the end is u - 8: 6.0e-4 -> 3.0e-4 against 64 bits at
+    // 8 x 4096, 12.8 -> 12.9 us (packed pairs).
+    uint32_t pw[2][2];   // fp16 pairs (heads 2c, 2c + 1)
+    F2 ps = f2_make(0.f, 0.f), pz = ps;
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < 2; ++u)
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          p[u][hf][e] = exp2_approx(sc[u][hf][e] - mnew);
-          ps += p[u][hf][e];
-          pz = fmaf(p[u][hf][e], zv[u][hf], pz);
-        }
-      l[e] = fmaf(l[e], corr[e], ps);
-      bs[e] = fmaf(bs[e], corr[e], pz);
-      m[e] = mnew;
+      for (int hf = 0; hf < 2; ++hf) {
+        const F2 p = f2_make(exp2_approx(sc[u][hf][0] - mnew[0]), exp2_approx(sc[u][hf][1] - mnew[1]));
+        float w0, w1;
+        f2_split(f2_mul(p, f2_make(wv[u][hf], wv[u][hf])), w0, w1);
+        pw[u][hf] = pack_half2_bits(w0, w1);
+        const float2 wr = __half22float2(*reinterpret_cast<const __half2*>(&pw[u][hf]));
+        ps = f2_add(ps, p);
+        pz = f2_fma(p, f2_make(zv[u][hf], zv[u][hf]), pz);
+        pz = f2_fma(f2_make(wr.x, wr.y), f2_make(m8r, m8r), pz);
+      }
+    float ps_e[2], pz_e[2];
+    f2_split(ps, ps_e[0], ps_e[1]);
+    f2_split(pz, pz_e[0], pz_e[1]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      l[e] = fmaf(l[e], corr[e], ps_e[e]);
+      bs[e] = fmaf(bs[e], corr[e], pz_e[e]);
     }
     if (__any_sync(0xffffffffu, moved)) {
 #pragma unroll
@@ -406,13 +424,12 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnCtasPerSm) attn_kernel(A
         o[mu][1] *= corr[1], o[mu][3] *= corr[1];
       }
     }
-    // ---- o^T += V^T P'^T with P' = p alpha' / r in fp16: the pairs (token,
-    // heads 2c, 2c+1) transposed to (head g, tokens 2c, 2c+1) are the B
-    // fragment (tokens 0..7 in register 0, 8..15 in register 1)
+    // ---- o^T += V^T P'^T: the pairs (token, heads 2c, 2c+1) transposed to
+    // (head g, tokens 2c, 2c+1) are the B fragment (tokens 0..7 in register 0,
+    // 8..15 in register 1)
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const uint32_t pb0 = transpose8x8(pack_half2_bits(p[u][0][0] * wv[u][0], p[u][0][1] * wv[u][0]));
-      const uint32_t pb1 = transpose8x8(pack_half2_bits(p[u][1][0] * wv[u][1], p[u][1][1] * wv[u][1]));
+      const uint32_t pb0 = transpose8x8(pw[u][0]), pb1 = transpose8x8(pw[u][1]);
       uint32_t vx[4][VW];
 #pragma unroll
       for (int rr = 0; rr < 4; ++rr) {
