@@ -618,24 +618,38 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(AttnArgs a, int nchun
   for (int i = 0; i < DPL; i += 2) *reinterpret_cast<__half2*>(out + i) = __floats2half2_rn(o[i] * inv, o[i + 1] * inv);
 }
 
-// CTAs per cluster and clusters per (batch, kv head).  Up to 8 chunks are one
-// cluster and one kernel.  Where the SMs would take more (few sequences), one
-// cluster of 8 stays ahead of several and their merge up to about 1024 tokens
-// per chunk: 32 query and 8 kv heads, D 128, lengths S / 2 to S, us,
-//                              1 x 8   2 x 8   4 x 8   8 x 8
-//   1 sequence,  S =  2048      5.25    7.2
-//   1 sequence,  S =  8192      8.9    10.2     9.5    10.3
-//   2 sequences, S = 16384     16.9    14.4    15.7
-//   1 sequence,  S = 32768     22.5             17.0    16.2
+// CTAs per cluster and clusters per (batch, kv head); n: the chunks that the
+// SMs take at once.  Up to 8 are one cluster and no second kernel.  Where the
+// SMs take more, one cluster of 8 stays ahead up to a length, beyond which the
+// slots it leaves empty cost more than the merge of several.  How the chunks
+// are cut then goes by how they fill the SMs: single CTAs always do, clusters
+// of 4, 6, 7 and 8 do nearly, of 3 and 5 do not, and one CTA too many on an SM
+// costs the more the longer the chunks are.  32 query and 8 kv heads, D 128, all
+// sequences S long, us, for one cluster of 8 / the cut between / single CTAs:
+//   S        n = 9 (B 8)       12 (B 6)            15 (B 5)            19 (B 4)
+//    8192    22.3 /  / 24.1    21.6 / 2x6 20.6 /   21.0 / 2x7 19.0 /   14.5 /  / 19.0
+//   16384    38.6 /  / 38.3    37.4 / 2x6 32.0 /   36.5 / 2x7 29.1 /   23.8 /  / 25.9
+//   32768    72.1 /  / 68.1    68.1 /  / 54.1      66.8 /  / 47.5      42.6 /  / 39.5
+//   65536     153 /  / 133      131 /  / 102        127 /  / 83.1      79.0 /  / 68.0
+// n = 25 (B 3): 16384 23.5 / 3x8 21.1 / 22.2, 65536 78.8 / / 54.3; n = 38
+// (B 2): 16384 22.8 / 2x8 17.2 / 23.3, 65536 77.6 / 9x4 39.5 / 44.3; n = 8 at 65536
+// (48 query and 12 kv heads, D 64): 110.5 / / 109.9, lengths S / 2 to S 94.1 / / 89.1.
 struct AttnPlan {
   int cluster, clusters;
 };
 
 AttnPlan plan_attention(int64_t B, int64_t S, int64_t Hkv) {
+  constexpr int kMax = kAttnMaxCluster;
   const int n = decode_attention_chunks(B, S, Hkv);
-  if (n <= kAttnMaxCluster) return {n, 1};
-  const int64_t by_len = (S + 1024 * kAttnMaxCluster - 1) / (1024 * kAttnMaxCluster);
-  return {kAttnMaxCluster, (int)(by_len < n / kAttnMaxCluster ? by_len : n / kAttnMaxCluster)};
+  if (n <= kMax) return S <= 40960 ? AttnPlan{n, 1} : AttnPlan{1, n};
+  if (n < 24) {
+    const int64_t one_up_to = n == 9 ? 12288 : n < 12 ? 8192 : n < 16 ? 6144 : n < 18 ? 8192 : 14336;
+    if (S <= one_up_to) return {kMax, 1};
+    return n >= 12 && n < 16 && S <= 24576 ? AttnPlan{n / 2, 2} : AttnPlan{1, n};
+  }
+  if (S > 24576 && n < 48) return n < 28 ? AttnPlan{1, n} : AttnPlan{4, n / 4};
+  const int64_t k = n < 32 && S > 10240 ? 3 : (S + 1024 * kMax - 1) / (1024 * kMax);   // 1024 tokens a chunk
+  return {kMax, (int)(k < n / kMax ? k : n / kMax)};
 }
 
 template <int D, int G>
