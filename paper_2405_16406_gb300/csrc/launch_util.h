@@ -48,13 +48,18 @@ cudaError_t prepare_launch(Kern kern, int threads, size_t smem, int* blocks_per_
     return cudaSuccess;
   }
   size_t& lim = limit[std::make_pair(dev, reinterpret_cast<const void*>(kern))];
-  if (smem > 48 * 1024 && smem > lim) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+  if (e != cudaSuccess) return e;
+  // the default limit of 48 KB holds for static and dynamic memory together
+  // (a row of 12288 floats is 48 KB by itself)
+  if (smem + fa.sharedSizeBytes > 48 * 1024 && smem > lim) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     lim = smem;
   }
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   occ[key] = per_sm;
