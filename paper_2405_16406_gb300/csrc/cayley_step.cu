@@ -505,8 +505,7 @@ cudaError_t launch_cayley_n(const CayleyArgs& a, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3((unsigned)a.batch), dim3(S::THREADS), S::BYTES, stream, 1, a.R, a.grad, a.alpha,
                  a.iters, a.R_out, a.Y_out);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int N, int C>
@@ -518,8 +517,7 @@ cudaError_t launch_cayley_cluster(const CayleyArgs& a, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3((unsigned)(a.batch * C)), dim3(L::THREADS), L::BYTES, stream, C, a.R, a.grad, a.alpha,
                  a.iters, a.R_out, a.Y_out);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 // Clusters of this kernel that can be resident at once, asked once per device

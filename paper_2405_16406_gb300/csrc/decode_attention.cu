@@ -666,9 +666,8 @@ cudaError_t launch_dg(const AttnArgs& a, cudaStream_t stream) {
   if (p.clusters > 1) {
     const int64_t groups = (a.B * a.Hq + 3) / 4;
     e = launch_pdl(attn_combine_kernel<D>, dim3((unsigned)groups), dim3(128), 0, stream, 1, a, p.clusters);
-    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return e;
 }
 
 template <int D>

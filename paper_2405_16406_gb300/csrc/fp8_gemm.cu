@@ -527,8 +527,7 @@ cudaError_t launch_t(const Fp8GemmArgs& a, cudaStream_t stream) {
   Fp8GemmParams p{a.a_scale, a.a_zero, a.w_scale, a.w_rowsum, a.y, a.acc_out, device_status_word(),
                   (int)a.M, (int)a.N, (int)a.K, (int)(planes * a.K / BK), take_debug_stall() ? 1 : 0, BN};
   e = launch_pdl(kern, dim3(grid), dim3(kThreads), kSmemBytes, stream, 1, tmA, tmB, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <bool W4A8, bool ASYM>
@@ -546,8 +545,7 @@ cudaError_t launch_pair_t(const Fp8GemmArgs& a, int bn, int clusters, cudaStream
   Fp8GemmParams p{a.a_scale, a.a_zero, a.w_scale, a.w_rowsum, a.y, a.acc_out, device_status_word(),
                   (int)a.M, (int)a.N, (int)a.K, (int)(planes * a.K / BK), take_debug_stall() ? 1 : 0, bn};
   e = launch_pdl(kern, dim3(grid), dim3(kThreads), kPairSmem, stream, 2, tmA, tmB, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 // Tile width of the pair kernel for a call, 0 for the single-CTA kernel (up to

@@ -28,6 +28,15 @@ inline int device_sm_count() {
   return cache[dev];
 }
 
+// A failed call also leaves its error in the thread's last-error slot.  It is
+// reported through the status of the call it belongs to, so it is taken out of
+// the slot, where the caller's next check would find it; nothing here reads the
+// slot, which may hold an error of the caller's own.
+inline cudaError_t take_error(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // Makes sure the kernel may use `smem` bytes of dynamic shared memory and
 // returns the number of resident blocks per SM for this launch shape (at
 // least 1).  The kernel's limit only ever grows (one kernel is launched with
@@ -50,17 +59,17 @@ cudaError_t prepare_launch(Kern kern, int threads, size_t smem, int* blocks_per_
   size_t& lim = limit[std::make_pair(dev, reinterpret_cast<const void*>(kern))];
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return take_error(e);
   // the default limit of 48 KB holds for static and dynamic memory together
   // (a row of 12288 floats is 48 KB by itself)
   if (smem + fa.sharedSizeBytes > 48 * 1024 && smem > lim) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return take_error(e);
     lim = smem;
   }
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return take_error(e);
   if (per_sm < 1) per_sm = 1;
   occ[key] = per_sm;
   *blocks_per_sm = per_sm;
@@ -145,7 +154,7 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
   }
   cfg.attrs = attr;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+  return take_error(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
 }
 
 }  // namespace spinq

@@ -375,8 +375,7 @@ cudaError_t launch_rows(Kern kern, int threads, size_t smem, const RotQuantArgs&
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   const int64_t grid = a.rows < cap ? a.rows : cap;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(threads), smem, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int LW, int L, bool SYM, bool CLAMP, bool SG>
@@ -414,8 +413,7 @@ cudaError_t launch_norot_for(const RotQuantArgs& a, cudaStream_t stream, bool* h
   cudaError_t e = prepare_launch(kern, threads, 0, &per_sm);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3((unsigned)a.rows), dim3(threads), 0, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

@@ -402,8 +402,7 @@ cudaError_t launch_plain(const KVArgs& a, cudaStream_t stream) {
   if (blocks < 1) blocks = 1;
   const cudaError_t e =
       launch_pdl(rotate_quant_kv_kernel<D, CLAMP>, dim3((unsigned)blocks), dim3(kWarps * 32), 0, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 // Head ranges for `tokens`: enough items for every resident warp, ranges long
@@ -446,8 +445,7 @@ cudaError_t launch_rope_w(const KVArgs& a, const RopePlan& plan, cudaStream_t st
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   if (blocks > cap) blocks = cap;
   e = launch_pdl(kern, dim3((unsigned)blocks), dim3(W * 32), smem, stream, 1, a, plan);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 // CTAs of 8 warps where every resident warp has work (2048 tokens of 48 heads:

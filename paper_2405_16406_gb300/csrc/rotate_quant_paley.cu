@@ -489,8 +489,7 @@ cudaError_t launch_paley(const RotQuantArgs& a, cudaStream_t stream) {
   RotQuantArgs la = a;
   la.debug_stall = take_debug_stall() ? 1 : 0;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(S::THREADS), S::BYTES, stream, 1, tmx, la);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int NS, bool SYM, bool CLAMP, bool SG>

@@ -128,8 +128,7 @@ cudaError_t launch_ns(const RotQuantArgs& a, cudaStream_t stream) {
   const int64_t cap = NS == 0 ? INT32_MAX : (int64_t)device_sm_count() * per_sm;
   const int64_t grid = a.rows < cap ? a.rows : cap;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(kThreads), smem, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <bool SYM, bool ROWSUM, bool CLAMP>

@@ -389,8 +389,7 @@ cudaError_t launch_t(const GemmArgs& a, int cluster, cudaStream_t stream) {
   p.a.debug_stall = take_debug_stall() ? 1 : 0;
   e = launch_pdl(kern, dim3((unsigned)cluster, (unsigned)((a.N + 127) / 128)), dim3(kThreads), smem, stream, cluster,
                  tmW, tmA, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <bool ASYM, bool ACC_OUT>

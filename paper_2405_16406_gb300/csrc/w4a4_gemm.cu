@@ -1107,8 +1107,7 @@ cudaError_t launch_tn(const GemmArgs& a, cudaStream_t stream) {
   la.debug_stall = take_debug_stall() ? 1 : 0;
   e = launch_pdl(kern, dim3(grid), dim3(kThreads), smem, stream, 1, tmA, tmB, la, (int)(a.K / 128), m_tiles,
                  tiles);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int MT, bool ASYM, bool ACC_OUT>
@@ -1144,8 +1143,7 @@ cudaError_t launch_dec_t(const GemmArgs& a, float* ws_acc, int* ws_cnt, int nspl
     return cudaErrorInvalidValue;
   dim3 grid((unsigned)nsplit, (unsigned)ntiles);
   e = launch_pdl(kern, grid, dim3(kDecThreads), L::dyn_bytes, stream, 1, tmW, tmA, a, ws_acc, ws_cnt, ksteps, nsplit);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int MN>

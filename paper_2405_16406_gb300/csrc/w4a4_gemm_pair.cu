@@ -585,8 +585,7 @@ cudaError_t launch_pair_t(const GemmArgs& a, cudaStream_t stream, bool* handled)
   *handled = true;
   e = launch_pdl(kern, dim3(2 * (unsigned)clusters), dim3(kThreads), L::dyn_bytes, stream, 2, tmA, tmB, tmY, a,
                  device_status_word(), (int)(a.K / 128), m_tiles, tiles);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

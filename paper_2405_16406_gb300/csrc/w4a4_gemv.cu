@@ -155,8 +155,7 @@ cudaError_t launch_gemv_t(const GemmArgs& a, cudaStream_t stream) {
   const int64_t by_n = (warps_needed + kGemvWarps - 1) / kGemvWarps;
   if (grid > by_n) grid = by_n;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(kGemvThreads), smem, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int MT>

@@ -544,8 +544,7 @@ cudaError_t launch_rs_t(const GemmArgs& a, cudaStream_t stream) {
   cudaError_t e = prepare_launch(kern, warps * 32, smem, &per_sm);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(warps * 32), smem, stream, 1, a, device_status_word());
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int NKW, int NT>
@@ -575,8 +574,7 @@ cudaError_t launch_tc_t(const GemmArgs& a, cudaStream_t stream) {
   cudaError_t e = prepare_launch(kern, wk * 32, smem, &per_sm);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3((unsigned)grid), dim3(wk * 32), smem, stream, 1, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int NT>
