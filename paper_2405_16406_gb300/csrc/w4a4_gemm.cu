@@ -1075,16 +1075,25 @@ bool encode_y_map(CUtensorMap* map, void* y, int64_t M, int64_t N) {
 
 namespace {
 
-// Width of 256-row tiles: 192 columns where they save work for whole waves.
-// us per tile: 0.66 per 128-deep K step + 5 for the epilogue at 256 columns,
-// 0.60 + 4 at 192 (a K step is bound by the unpack warps, 512 rows against 448).
-// 1531 x 4096 -> 14336 81.7 us at 256, 72.3 at 192 (3 waves of either); 512 x
-// 4096 -> 4096 28.5 and 25.5 (one); 2048 x 14336 -> 4096 81.3 and 143 (one, two).
-int tile256_width(int64_t M, int64_t N, int64_t K, int64_t sms) {
-  const int64_t m_tiles = (M + 255) / 256, ks = K / 128;
-  const double wide = (double)((m_tiles * ((N + BN - 1) / BN) + sms - 1) / sms) * (0.66 * (double)ks + 5.0);
-  const double slim = (double)((m_tiles * ((N + 191) / 192) + sms - 1) / sms) * (0.60 * (double)ks + 4.0);
-  return slim < wide ? 192 : BN;
+// Width of the 256-row tiles of a call and the time that choose_prefill
+// expects of them (us): 192 columns where they save work for whole waves.
+// Per tile 0.66 us a 128-deep K step + 5 for the epilogue (the single
+// accumulator buffer serialises it, all unpack warps share it) at 256 columns,
+// 0.60 + 4 at 192 (a K step is bound by the unpack warps, 512 rows against 448),
+// and 4.9 us once.  Automatic choice, 256 columns only -> with this rule:
+// 512 x 4096 -> 14336 30.1 -> 28.7 us, 1280 x 14336 -> 4096 83.1 -> 79.1,
+// 1531 x 4096 -> 4096 29.7 -> 28.1; 768 x 3072 -> 8192 27.6 (SM pairs) -> 22.7.
+struct Tile256 {
+  int width;
+  double us;
+};
+
+Tile256 tile256(int64_t M, int64_t N, int64_t K, int64_t sms) {
+  const int64_t m_tiles = (M + 255) / 256;
+  const double ks = (double)(K / 128);
+  const double wide = (double)((m_tiles * ((N + BN - 1) / BN) + sms - 1) / sms) * (0.66 * ks + 5.0);
+  const double slim = (double)((m_tiles * ((N + 191) / 192) + sms - 1) / sms) * (0.60 * ks + 4.0);
+  return slim < wide ? Tile256{192, slim + 4.9} : Tile256{BN, wide + 4.9};
 }
 
 template <int MT, bool ASYM, bool ACC_OUT, int TN>
@@ -1113,8 +1122,7 @@ cudaError_t launch_tn(const GemmArgs& a, cudaStream_t stream) {
 template <int MT, bool ASYM, bool ACC_OUT>
 cudaError_t launch_t(const GemmArgs& a, cudaStream_t stream) {
   if constexpr (MT == 2) {
-    if (tile256_width(a.M, a.N, a.K, device_sm_count()) == 192)
-      return launch_tn<MT, ASYM, ACC_OUT, 192>(a, stream);
+    if (tile256(a.M, a.N, a.K, device_sm_count()).width == 192) return launch_tn<MT, ASYM, ACC_OUT, 192>(a, stream);
   }
   return launch_tn<MT, ASYM, ACC_OUT, BN>(a, stream);
 }
@@ -1196,9 +1204,7 @@ namespace {
 // A persistent CTA (or SM pair) runs ceil(tiles / CTAs) tiles back to back:
 //   128 x 256 tiles, one CTA:  0.485 us per 128-deep K step + 3 us (the
 //     epilogue overlaps the next tile);
-//   256 x 256 tiles, one CTA:  0.66 us per K step + 5.0 us per tile (the
-//     single accumulator buffer serialises the epilogue, which all unpack
-//     warps share) + 4.9 us once;
+//   256-row tiles, one CTA:  tile256 above, at the width the launch takes;
 //   256 x 256 tiles, SM pair:  0.45 us per K step, epilogue overlapped,
 //     + 3 us for the last tile's epilogue.
 struct PrefillChoice {
@@ -1211,7 +1217,7 @@ PrefillChoice choose_prefill(int64_t M, int64_t N, int64_t K, bool allow_pair) {
   const int64_t sms = device_sm_count(), ks = K / 128;
   const int64_t tiles256 = ((M + 255) / 256) * ((N + BN - 1) / BN);
   const int64_t tiles128 = ((M + 127) / 128) * ((N + BN - 1) / BN);
-  const double est256 = (double)((tiles256 + sms - 1) / sms) * (0.66 * (double)ks + 5.0) + 4.9;
+  const double est256 = tile256(M, N, K, sms).us;
   const double est128 = (double)((tiles128 + sms - 1) / sms) * (0.485 * (double)ks + 3.0);
   PrefillChoice c = est256 < est128 ? PrefillChoice{SPINQ_GEMM_TILE256, est256} : PrefillChoice{SPINQ_GEMM_TILE128, est128};
   if (pairs > 0) {
