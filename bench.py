@@ -697,7 +697,8 @@ def run_configs(dev, hbm_peak, fp8_peak):
               "frac_hbm": round(rq_bytes / rq_us / 1e3 / hbm_peak, 4)}
         gm = {"us": round(g_us, 3), "tops": round(ops / g_us / 1e6, 1),
               "kernel_plan": spinq.spinq_w4a4_gemm_splitk_plan(Mr, Nr, Kr) if Mr <= 256
-              else spinq.spinq_w4a4_gemm_plan(Mr, Nr, Kr)}
+              else spinq.spinq_w4a4_gemm_plan(Mr, Nr, Kr),
+              "cluster": spinq.spinq_w4a4_gemm_cluster_plan(Mr, Nr, Kr) if Mr <= 256 else 0}
         if gemm_bound == "tensor":
             gm["frac_e4m3"] = round(ops / g_us / 1e6 / fp8_peak, 4)
         else:

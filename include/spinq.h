@@ -178,7 +178,8 @@ int64_t spinq_w4a4_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K);
  * the outputs itself and no workspace is used).  Under the automatic choice
  * (no kernel and no number of slices selected) most calls of up to 128 tokens
  * instead take clusters of up to 8 CTAs per 128 channels that sum their slices
- * over distributed shared memory; `workspace` is then checked but not touched.  For M > 256 the call runs
+ * over distributed shared memory (spinq_w4a4_gemm_cluster_plan, spinq_gemm_cluster);
+ * `workspace` is then checked but not touched.  For M > 256 the call runs
  * the same kernel as spinq_w4a4_gemm and does not touch `workspace`.
  *   workspace       device buffer of spinq_w4a4_gemm_workspace_bytes(M, N, K)
  *                   bytes, 16-byte aligned, all zero before the first call;
@@ -323,6 +324,18 @@ int spinq_gemm_select_kernel(int kernel);
 int spinq_gemm_split_k(int n);
 
 /*
+ * spinq_gemm_cluster -- process-wide number of CTAs per cluster of the
+ * clustered decode kernel (spinq_w4a4_gemm_splitk / _noalloc, M <= 128): 1..8
+ * fixes it (at most K / 128) and gives the kernel every call it serves while no
+ * other kernel (spinq_gemm_select_kernel) and no number of K slices
+ * (spinq_gemm_split_k) is selected; 0 lets the cost model decide (the default).
+ * A tuning and testing control; workspaces keep their size and are checked as
+ * before.  Returns the previous value, or -1 (and changes nothing) for a value
+ * out of range.
+ */
+int spinq_gemm_cluster(int n);
+
+/*
  * spinq_w4a4_gemm_plan -- the kernel (SPINQ_GEMM_TILE128, _TILE256, _PAIR,
  * _GEMV or _TCGEMV) that spinq_w4a4_gemm runs for an M x N x K call on the current CUDA
  * device under the current selection; -1 for shapes the call rejects.
@@ -331,16 +344,24 @@ int spinq_gemm_split_k(int n);
 int spinq_w4a4_gemm_plan(int64_t M, int64_t N, int64_t K);
 
 /*
- * spinq_w4a4_gemm_splitk_plan -- the kernel that spinq_w4a4_gemm_splitk runs
- * for an M x N x K call given a workspace of spinq_w4a4_gemm_workspace_bytes
- * bytes, before the choice of clusters described there (which needs none and
- * keeps this answer, so that workspaces sized by it stay valid):
+ * spinq_w4a4_gemm_splitk_plan -- the kernel that spinq_w4a4_gemm_splitk sizes
+ * its workspace for and, where spinq_w4a4_gemm_cluster_plan is 0, runs for an
+ * M x N x K call given a workspace of spinq_w4a4_gemm_workspace_bytes bytes:
  * SPINQ_GEMM_SPLITK, with *nsplit (may be NULL) set to its number of K
  * slices per 128-channel tile (1: no slicing, no workspace), or the kernel
  * spinq_w4a4_gemm would run (*nsplit = 0).  -1 for shapes the call rejects.
  * Launches nothing.
  */
 int spinq_w4a4_gemm_splitk_plan(int64_t M, int64_t N, int64_t K, int* nsplit);
+
+/*
+ * spinq_w4a4_gemm_cluster_plan -- the CTAs per cluster with which the clustered
+ * decode kernel serves spinq_w4a4_gemm_splitk for an M x N x K call (given such
+ * a workspace) on the current CUDA device under the current selection; 0 where
+ * the kernel of spinq_w4a4_gemm_splitk_plan serves it, -1 for shapes the call
+ * rejects.  Launches nothing.
+ */
+int spinq_w4a4_gemm_cluster_plan(int64_t M, int64_t N, int64_t K);
 
 /*
  * spinq_rope_rotate_quant_kv -- spinq_rotate_quant_kv with the rotary

@@ -434,6 +434,8 @@ int spinq_gemm_select_kernel(int kernel) { return w4a4_gemm_select(kernel); }
 
 int spinq_gemm_split_k(int n) { return w4a4_gemm_split_k(n); }
 
+int spinq_gemm_cluster(int n) { return w4a4_gemm_cluster(n); }
+
 int spinq_w4a4_gemm_plan(int64_t M, int64_t N, int64_t K) {
   if (M <= 0 || N <= 0 || K <= 0 || K % 128 != 0 || N % 16 != 0) return -1;
   return plan_w4a4_gemm(M, N, K);
@@ -446,6 +448,11 @@ int spinq_w4a4_gemm_splitk_plan(int64_t M, int64_t N, int64_t K, int* nsplit) {
   const int kind = plan_w4a4_gemm_splitk(M, N, K, &ns);
   if (nsplit) *nsplit = ns;
   return kind;
+}
+
+int spinq_w4a4_gemm_cluster_plan(int64_t M, int64_t N, int64_t K) {
+  if (M <= 0 || N <= 0 || K <= 0 || K % 128 != 0 || N % 16 != 0 || K > 65536) return -1;
+  return plan_w4a4_gemm_cluster(M, N, K);
 }
 
 spinq_status spinq_device_status(int32_t* detail) {

@@ -263,6 +263,10 @@ int w4a4_gemm_select(int kernel);
 // Process-wide fixed count of the split-K kernel's K slices (0: the cost
 // model picks).
 int w4a4_gemm_split_k(int n);
+// 0: the cost model, 1..kDecodeMaxCluster: that cluster size.
+int w4a4_gemm_cluster(int n);
+// Cluster size with which the split-K entry point runs the clustered kernel, 0 for another kernel.
+int plan_w4a4_gemm_cluster(int64_t M, int64_t N, int64_t K);
 // The prefill kernel (SPINQ_GEMM_TILE128 / TILE256 / PAIR) launch_w4a4_gemm
 // runs for this shape on the current device.
 int plan_w4a4_gemm(int64_t M, int64_t N, int64_t K);

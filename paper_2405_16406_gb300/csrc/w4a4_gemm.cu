@@ -1197,6 +1197,13 @@ int w4a4_gemm_split_k(int n) {
   return g_split_k.exchange(n);
 }
 
+std::atomic<int> g_cluster{0};
+
+int w4a4_gemm_cluster(int n) {
+  if (n < 0 || n > kDecodeMaxCluster) return -1;
+  return g_cluster.exchange(n);
+}
+
 namespace {
 
 // Kernel and tile height from a wave-quantised cost model (microseconds,
@@ -1354,6 +1361,19 @@ DecodePlan plan_splitk_entry(int64_t M, int64_t N, int64_t K, bool room) {
   return plan_decode(M, N, K, lo, hi, g_gemm_kernel.load(std::memory_order_relaxed) != SPINQ_GEMM_SPLITK);
 }
 
+// The clustered kernel serves the shape and no other kernel is selected.
+bool cluster_allowed(int64_t M, int64_t N) {
+  return M <= kDecodeClusterMaxM && (N + 127) / 128 <= 65535 &&
+         g_gemm_kernel.load(std::memory_order_relaxed) == SPINQ_GEMM_AUTO &&
+         g_split_k.load(std::memory_order_relaxed) == 0;
+}
+
+// The selected cluster size for a call, 0 if none is selected or none fits.
+int fixed_cluster(int64_t M, int64_t N, int64_t K) {
+  const int c = (int)std::min<int64_t>(g_cluster.load(std::memory_order_relaxed), K / 128);
+  return c > 0 && cluster_allowed(M, N) && w4a4_decode_clusters(c) > 0 ? c : 0;
+}
+
 // Cluster size with which the clustered kernel (w4a4_decode_cluster.cu) takes
 // a call of up to 128 tokens under the automatic choice, 0 where the plan's
 // route (`other_us`) is predicted to be as fast.  Microseconds, fitted on GB300
@@ -1372,9 +1392,7 @@ DecodePlan plan_splitk_entry(int64_t M, int64_t N, int64_t K, bool room) {
 // microsecond: below that lie calls of a few K steps, where start-up is all
 // there is (24 tokens, 256 -> 512: 5.8 against 6.4).
 int decode_cluster(int64_t M, int64_t N, int64_t K, double other_us) {
-  if (M > kDecodeClusterMaxM || g_gemm_kernel.load(std::memory_order_relaxed) != SPINQ_GEMM_AUTO ||
-      g_split_k.load(std::memory_order_relaxed) != 0)
-    return 0;
+  if (!cluster_allowed(M, N)) return 0;
   const int64_t tiles = (N + 127) / 128, ks = K / 128;
   const double step = 0.27 + 0.0018 * (double)((M + 15) / 16 * 16);
   int best = 0;
@@ -1417,10 +1435,17 @@ int plan_w4a4_gemm_splitk(int64_t M, int64_t N, int64_t K, int* nsplit) {
   return SPINQ_GEMM_SPLITK;
 }
 
+int plan_w4a4_gemm_cluster(int64_t M, int64_t N, int64_t K) {
+  if (const int c = fixed_cluster(M, N, K)) return c;
+  if (M > kDecodeClusterMaxM || tcgemv_serves(M, N, K) || gemv_serves(M, K)) return 0;
+  return decode_cluster(M, N, K, plan_splitk_entry(M, N, K, true).us);
+}
+
 cudaError_t launch_w4a4_gemm_splitk(const GemmArgs& a, void* workspace, int64_t workspace_bytes,
                                     cudaStream_t stream) {
   if (a.M == 0 || a.N == 0) return cudaSuccess;
   if (a.M > kDecodeMaxM) return launch_w4a4_gemm(a, stream);
+  if (const int c = fixed_cluster(a.M, a.N, a.K)) return launch_w4a4_decode_cluster(a, c, stream);
   if (tcgemv_serves(a.M, a.N, a.K)) {
     bool handled = false;
     const cudaError_t et = launch_w4a4_gemv_tc(a, stream, &handled);

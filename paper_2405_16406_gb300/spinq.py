@@ -38,6 +38,7 @@ EXPORTED = (
     "spinq_rotate_quant_act", "spinq_quant_weight", "spinq_w4a4_gemm", "spinq_rotate_quant_kv",
     "spinq_status_string", "spinq_device_status", "spinq_version", "spinq_w4a4_gemm_workspace_bytes",
     "spinq_w4a4_gemm_splitk", "spinq_w4a4_gemm_noalloc", "spinq_gemm_select_kernel", "spinq_gemm_split_k",
+    "spinq_gemm_cluster", "spinq_w4a4_gemm_cluster_plan",
     "spinq_w4a4_gemm_plan", "spinq_w4a4_gemm_splitk_plan", "spinq_cayley_step",
     "spinq_rotate_quant_act8", "spinq_quant_weight8", "spinq_fp8_gemm", "spinq_w4a8_gemm",
     "spinq_rope_rotate_quant_kv", "spinq_decode_attention_workspace_bytes", "spinq_decode_attention_kv4",
@@ -90,6 +91,10 @@ _lib.spinq_gemm_select_kernel.restype = ctypes.c_int
 _lib.spinq_gemm_select_kernel.argtypes = [ctypes.c_int]
 _lib.spinq_gemm_split_k.restype = ctypes.c_int
 _lib.spinq_gemm_split_k.argtypes = [ctypes.c_int]
+_lib.spinq_gemm_cluster.restype = ctypes.c_int
+_lib.spinq_gemm_cluster.argtypes = [ctypes.c_int]
+_lib.spinq_w4a4_gemm_cluster_plan.restype = ctypes.c_int
+_lib.spinq_w4a4_gemm_cluster_plan.argtypes = [_I64, _I64, _I64]
 _lib.spinq_w4a4_gemm_plan.restype = ctypes.c_int
 _lib.spinq_w4a4_gemm_plan.argtypes = [_I64, _I64, _I64]
 _lib.spinq_w4a4_gemm_splitk_plan.restype = ctypes.c_int
@@ -252,12 +257,22 @@ def spinq_gemm_split_k(n: int) -> int:
     return int(_lib.spinq_gemm_split_k(n))
 
 
+def spinq_gemm_cluster(n: int) -> int:
+    return int(_lib.spinq_gemm_cluster(n))
+
+
+def spinq_w4a4_gemm_cluster_plan(M: int, N: int, K: int) -> int:
+    """CTAs per cluster of the clustered kernel where it serves spinq_w4a4_gemm_splitk, else 0."""
+    return int(_lib.spinq_w4a4_gemm_cluster_plan(M, N, K))
+
+
 def spinq_w4a4_gemm_plan(M: int, N: int, K: int) -> int:
     return int(_lib.spinq_w4a4_gemm_plan(M, N, K))
 
 
 def spinq_w4a4_gemm_splitk_plan(M: int, N: int, K: int) -> tuple:
-    """(kernel, K slices) of spinq_w4a4_gemm_splitk for an M x N x K call."""
+    """(kernel, K slices) of spinq_w4a4_gemm_splitk for an M x N x K call where
+    spinq_w4a4_gemm_cluster_plan is 0."""
     ns = ctypes.c_int(0)
     kind = int(_lib.spinq_w4a4_gemm_splitk_plan(M, N, K, ctypes.byref(ns)))
     return kind, int(ns.value)
