@@ -219,12 +219,13 @@ spinq_status spinq_w4a4_gemm_splitk(const uint8_t* a_codes, const float* a_scale
  *   The call itself allocates nothing: no cudaMalloc/cudaFree and no
  *   allocating library routine.  It clears the part of the array it uses
  *   (cudaMemsetAsync on `stream`) before the kernel, since the array keeps
- *   the previous call's contents.
- *   The first call in each CUDA context looks up the array's device address
- *   (cudaGetSymbolAddress, with that device current) and caches it for that
- *   context; make that first call outside any stream capture.
- *   Every call shares the one array per device: calls that may overlap on the
- *   GPU (different streams without ordering between them) race on it.
+ *   the previous call's contents.  Calls that the clustered kernel serves
+ *   (spinq_w4a4_gemm_cluster_plan) use none of it and enqueue the kernel alone.
+ *   The first call in each CUDA context that uses the array looks up its device
+ *   address (cudaGetSymbolAddress, with that device current) and caches it for
+ *   that context; make that first call outside any stream capture.
+ *   The calls that use it share the one array per device: those that may overlap
+ *   on the GPU (different streams without ordering between them) race on it.
  */
 spinq_status spinq_w4a4_gemm_noalloc(const uint8_t* a_codes, const float* a_scale, const float* a_zero,
                                      const uint8_t* w_codes, const float* w_scale,

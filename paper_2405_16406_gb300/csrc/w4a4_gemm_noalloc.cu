@@ -102,15 +102,19 @@ extern "C" spinq_status spinq_w4a4_gemm_noalloc(const uint8_t* a_codes, const fl
   const int64_t need = spinq::w4a4_gemm_workspace_bytes(M, N, K);
   if (need > kNoAllocScratchBytes) return SPINQ_ESCRATCH;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const spinq::GemmArgs g{a_codes, a_scale, a_zero, w_codes, w_scale, w_rowsum, M, N, K, y_f16, acc_out};
+  // the clustered kernel sums in its own shared memory: nothing to clear, and
+  // the array stays free for other calls
+  const int cluster = spinq::plan_w4a4_gemm_cluster(M, N, K);
   void* ws = nullptr;
-  if (need > 0) {
+  if (need > 0 && cluster == 0) {
     if (scratch_address(&ws) != cudaSuccess) return SPINQ_ECUDA;
     // the array still holds what the previous call left in it: the partial
     // accumulators and tile counters must start at zero
     if (cudaMemsetAsync(ws, 0, (size_t)need, s) != cudaSuccess) return SPINQ_ECUDA;
   }
-  const spinq::GemmArgs g{a_codes, a_scale, a_zero, w_codes, w_scale, w_rowsum, M, N, K, y_f16, acc_out};
-  const cudaError_t e = spinq::launch_w4a4_gemm_splitk(g, ws, need, s);
+  const cudaError_t e = cluster > 0 ? spinq::launch_w4a4_decode_cluster(g, cluster, s)
+                                    : spinq::launch_w4a4_gemm_splitk(g, ws, need, s);
   if (e == cudaSuccess) return SPINQ_OK;
   return e == cudaErrorNotSupported ? SPINQ_EUNSUPPORTED : SPINQ_ECUDA;
 }
