@@ -298,8 +298,13 @@ spinq_status spinq_rotate_quant_kv(const void* q_in, void* q_out, const void* k_
  *                       into registers; else a CTA per 16 output channels
  *                       that stages them through shared memory; calls it
  *                       cannot serve use AUTO.
- * All kernels compute bit-identical outputs; this is a tuning and testing
- * control.  Returns the previous selection, or -1 (and changes nothing) for
+ * All kernels compute the same exact accumulators.  The outputs are
+ * bit-identical among TILE128, TILE256 and PAIR, whose epilogue takes the sums
+ * of the unsigned codes (s_n fma(alpha 2^18, S, c + d rowsum_n), fp32), and
+ * among GEMV, TCGEMV, SPLITK and the clustered kernel, whose epilogue takes the
+ * accumulator (s_n fma(alpha, acc, beta' rowsum_n)); between the two they may
+ * differ by fp32 roundings of 2^-24 s_n alpha sum_k u_a u_w.  This is a tuning
+ * and testing control.  Returns the previous selection, or -1 (and changes nothing) for
  * an unknown value.  Not synchronized with GEMM calls in other threads.
  */
 typedef enum {

@@ -188,8 +188,9 @@ struct Cfg {
 // null) after its last read.
 //   y = s_n (alpha (S - 8 rs_a - 8 rw_n) + beta' rw_n), S = acc * 2^18,
 //   evaluated as y = s_n * fma(alpha * 2^18, acc, c + d * rw_n) with
-//   c = -8 alpha rs_a and d = beta' - 8 alpha (the roundings of the other
-//   kernels, so that every kernel gives the same bits).
+//   c = -8 alpha rs_a and d = beta' - 8 alpha (the roundings of the
+//   128-row tiles and the SM pair, so that these kernels give the same bits; the
+//   decode kernels round on the accumulator instead).
 template <int TN, bool ASYM, bool ACC_OUT>
 __device__ __forceinline__ void epi256_share(const GemmArgs& args, uint32_t tq, int q, int lane, int part,
                                              int nparts, int64_t m_tile0, int64_t n0, const float* col_s,

@@ -39,8 +39,8 @@
 // Codes are made unsigned as in the other kernels (u = code ^ 8 for two's
 // complement codes, u = code for asymmetric activations), so
 //   acc = S - 8 sum_k u_a - 8 sum_k u_w + 64 K = S - 8 sum_k u_a - 8 rowsum_n
-// with S = sum_k u_a u_w.  The epilogue is the one of the other kernels, so
-// the outputs are bit-identical.
+// with S = sum_k u_a u_w.  The epilogue is the one of the other decode kernels,
+// so their outputs are bit-identical.
 #include <cuda_fp16.h>
 
 #include <utility>
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32) w4a4_gemv_tc_kernel(GemmArgs
 // A tile's K blocks meet in shared memory: each warp adds its exact partial
 // sums (as integers) into one of kRsSlots slots and arrives on the slot's
 // `full` barrier; the tile's epilogue warp (tiles w, w + W, ... go to warp w)
-// waits on it, applies the epilogue of the other kernels (bit-identical
+// waits on it, applies the epilogue of the other decode kernels (bit-identical
 // outputs), clears the slot and arrives on `empty`, which a warp waits on
 // before it adds tile ti + kRsSlots into the same slot.  Every wait is
 // bounded; one that gives up records SPINQ_ETIMEOUT and every warp leaves at
