@@ -39,7 +39,8 @@ namespace {
 
 template <int N>
 struct CayleyShape {
-  static constexpr int TR = N >= 128 ? 4 : (N >= 64 ? 2 : 1);  // rows per thread
+  static_assert(N == 16 || N == 128, "the other sizes take cayley_cluster_kernel");
+  static constexpr int TR = N == 128 ? 4 : 1;                   // rows per thread
   static constexpr int CG = N / 8;                              // column groups of 8
   static constexpr int RG = N / TR;                             // row groups
   static constexpr int THREADS = CG * RG;
@@ -74,9 +75,6 @@ __device__ __forceinline__ void mm_acc(const float* X, const float* B, int i0, i
         if constexpr (S::TR == 4) {
           const float4 t = *reinterpret_cast<const float4*>(X + k * S::S + i0);
           xv[q][0] = t.x, xv[q][1] = t.y, xv[q][2] = t.z, xv[q][3] = t.w;
-        } else if constexpr (S::TR == 2) {
-          const float2 t = *reinterpret_cast<const float2*>(X + k * S::S + i0);
-          xv[q][0] = t.x, xv[q][1] = t.y;
         } else {
           xv[q][0] = X[k * S::S + i0];
         }

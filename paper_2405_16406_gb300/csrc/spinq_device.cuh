@@ -18,17 +18,7 @@ namespace spinq {
 // D fragment: d[0..1] = (row g, n 2c..2c+1), d[2..3] = (row g+8, n 2c..2c+1)
 // with g = lane / 4, c = lane % 4.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void mma_16816_f16_f32(float d[4], const uint32_t a[4], uint32_t b0,
-                                                  uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%10,%11,%12,%13};\n"
-      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f), "f"(0.f),
-        "f"(0.f), "f"(0.f));
-}
-
-// Same MMA accumulating into d (C = D).
+// Accumulates into d (C = D).
 __device__ __forceinline__ void mma_16816_f16_f32_acc(float d[4], const uint32_t a[4], uint32_t b0,
                                                       uint32_t b1) {
   asm volatile(
