@@ -906,7 +906,7 @@ def variant8_records(dev, hbm_peak, fp8_peak):
                                             "rq_paley_kernel (int8 planes epilogue)")},
                 "gemm": {"us": round(g_us, 2), "tops": round(ops / g_us / 1e6, 1),
                          "tensor_frac_e4m3": round(planes * ops / g_us / 1e6 / fp8_peak, 4),
-                         "kernel": "fp8_gemm_kernel" + (" (two activation planes, K' = 2K)" if planes == 2 else "")},
+                         "kernel": "fp8_gemm_pair_kernel" + (" (two activation planes, K' = 2K)" if planes == 2 else "")},
                 "checked": "4 rows x 256 columns of the timed output vs the oracle's product of the same codes"}
             del outs, ys, wq
             torch.cuda.empty_cache()
@@ -1064,7 +1064,8 @@ def relaunch(args_n):
 
 
 PROFILE_CASES = ("attention", "rope_kv", "fp8_gemm", "w4a8_gemm", "rq8_paley", "cayley", "paley", "gemm",
-                 "gemm_gate_up", "decode_gemm", "decode_gemm16", "rq_h8192", "kv2048", "act_quant")
+                 "gemm_gate_up", "decode_gemm", "decode_gemm16", "rq_h8192", "kv2048", "act_quant",
+                 "decode_cluster", "weight_rows", "cayley32")
 
 
 def profile_case(name, reps):
@@ -1083,7 +1084,9 @@ def profile_case(name, reps):
     rq_h8192: the 4-bit R4 kernel with H8192 on 8192 x 8192 (asymmetric);
     kv2048: R3 + KV4 on the step's 2048 tokens (32 / 8 heads, D 128);
     act_quant: the step's gate_up activation quantizer (2048 x 4096, no
-    rotation, asymmetric)."""
+    rotation, asymmetric); decode_cluster: 77 tokens through 4096 -> 4096 on
+    the automatic route; weight_rows: 4096 x 14336 weights merged with
+    H28 x H512; cayley32: 32 rotations of 128 x 128, 2 iterations."""
     import numpy as np
     import torch
 
@@ -1152,11 +1155,20 @@ def profile_case(name, reps):
         c = synth.llama3_8b_gate_up()
         x = torch.from_numpy(c.x).to(dev)
         fn = lambda: spinq.rotate_quant_act(x, None, False)
-    elif name == "cayley":
+    elif name == "decode_cluster":
         rng = np.random.default_rng(0)
-        R = np.stack([np.linalg.qr(rng.standard_normal((128, 128)))[0] for _ in range(152)]).astype(np.float32)
+        qa = spinq.rotate_quant_act(torch.from_numpy(synth.activations(rng, 77, 4096)).to(dev), None)
+        qw = spinq.quant_weight(torch.from_numpy(synth.weights(rng, 4096, 4096)).to(dev), None)
+        fn = lambda: spinq.w4a4_gemm_splitk(qa, qw)
+    elif name == "weight_rows":
+        w = torch.from_numpy(synth.llama3_8b_down_proj().w).to(dev)
+        fn = lambda: spinq.quant_weight(w, (28, 512))
+    elif name in ("cayley", "cayley32"):
+        n = 32 if name == "cayley32" else 152
+        rng = np.random.default_rng(0)
+        R = np.stack([np.linalg.qr(rng.standard_normal((128, 128)))[0] for _ in range(n)]).astype(np.float32)
         Rt = torch.from_numpy(R).to(dev)
-        G = torch.from_numpy((rng.standard_normal((152, 128, 128)) * 0.5).astype(np.float32)).to(dev)
+        G = torch.from_numpy((rng.standard_normal((n, 128, 128)) * 0.5).astype(np.float32)).to(dev)
         fn = lambda: spinq.cayley_step(Rt, G, 0.01, 2)
     else:
         raise ValueError(f"unknown profile case {name}")

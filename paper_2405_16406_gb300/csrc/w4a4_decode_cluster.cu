@@ -24,8 +24,8 @@
 // kernel of w4a4_gemm.cu adds its partial sums by atomics in global memory and
 // lets the last slice of a tile convert them, 1.8 + 0.089 M us; over the
 // cluster that part is one pass over shared memory.  77 tokens, 4096 -> 4096,
-// with the quantizer: 22.7 us there, 11.7 here (clusters of 4); 14336 -> 4096:
-// 36.3 and 21.4 (30 MB, 4.3 us of HBM).  The row sum correction takes
+// with the quantizer: 23.0 us there, 11.6 here (clusters of 4); 14336 -> 4096:
+// 35.1 and 20.3 (30 MB, 4.3 us of HBM).  The row sum correction takes
 // w_rowsum instead of counting the weights again, which leaves their unpacking
 // to masks and stores.
 #include <cuda.h>

@@ -1383,15 +1383,17 @@ int fixed_cluster(int64_t M, int64_t N, int64_t K) {
 //   waves (4.3 + 0.021 M + steps (0.27 + 0.0018 MN)),
 // steps the 128-deep K steps of a CTA.  Measured with the activation quantizer
 // before it (graphs over rotating weights), the plan's route -> this one:
-//   24 tokens:  4096 -> 4096 11.6 -> 9.3 us, 14336 -> 4096 18.8 -> 17.6
-//   77 tokens:  4096 -> 4096 22.5 -> 11.7, 4096 -> 6144 23.5 -> 14.9,
-//               14336 -> 4096 36.3 -> 21.5, 3072 -> 16384 21.1 -> 19.3
-//   128 tokens: 8192 -> 3072 30.0 -> 17.7
+//   24 tokens:  4096 -> 4096 11.8 -> 9.5 us, 3072 -> 16384 17.5 -> 14.7
+//   77 tokens:  4096 -> 4096 23.0 -> 11.6, 4096 -> 6144 23.5 -> 14.7,
+//               14336 -> 4096 35.1 -> 20.3, 3072 -> 16384 20.2 -> 18.5
+//   128 tokens: 8192 -> 3072 30.5 -> 16.0
 // and the plan's route stays ahead where the tiles need a second wave (4096 ->
-// 28672 at 77 tokens, 128-row tiles: 26.4 against 33.8) and for wide outputs
-// at 128 tokens (3072 -> 16384: 21.9 against 23.0).  It has to win by half a
+// 28672 at 77 tokens, 128-row tiles: 25.6 against 40.8) and for wide outputs
+// at 128 tokens (3072 -> 16384: 21.1 against 22.4).  It has to win by half a
 // microsecond: below that lie calls of a few K steps, where start-up is all
-// there is (24 tokens, 256 -> 512: 5.8 against 6.4).
+// there is (24 tokens, 256 -> 512: 5.5 against 5.9).  The model is too dear for
+// long K at few tokens (24 tokens, 14336 -> 4096: stays at 18.4, clusters of 4
+// take 16.4).
 int decode_cluster(int64_t M, int64_t N, int64_t K, double other_us) {
   if (!cluster_allowed(M, N)) return 0;
   const int64_t tiles = (N + 127) / 128, ks = K / 128;
